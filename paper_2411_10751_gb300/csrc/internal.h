@@ -94,13 +94,12 @@ struct StepArgs {
   float* aux_wr;
 };
 
-// Arguments of the wall-bounded D2Q37 step (walls.cu): moments and collide
-// launches of one step.
+// Arguments of the wall-bounded D2Q37 step and moments readout (walls.cu).
 struct WallArgs {
   const void* fin;        // post-collision state of step t - 1, [Q][N]
   void* fout;             // collide: state written by this step
   const float* mprev;     // [4][N] rho, u_x, u_y, theta - 1 of the previous step (completed)
-  float* mcur;            // moments: this step's [4][N] (may be null); collide: read for grad theta
+  float* mcur;            // step: this step's [4][N] moments, written
   float* rho_out;         // moments readout (may be null)
   float* u_out;
   float* theta_out;
@@ -113,11 +112,12 @@ struct WallArgs {
   float rho0;
   float omega, beta;
   float h_coef;           // 1 - 1/Pr (H_i)
-  float wall_u[2][2];     // velocity of the bottom (0) and top (1) wall
-  float wall_tb[2];       // their temperature minus 1
+  double wall_u[2][2];    // velocity of the bottom (0) and top (1) wall (FP32 values; the completion is FP64)
+  double wall_tb[2];      // their temperature minus 1
   float tb_ref;           // reference temperature of the stored deviations minus 1
   float e_ref;            // rho0 D c0^2 tb_ref: energy moment of the reference offset
-  float* comp;            // completed unknowns of the six wall rows, [6][37][nx] (slot 3 side + r)
+  const float* comp;      // completed unknowns of the six wall rows, [6][37][nx] (slot 3 side + r)
+  float* comp_next;       // those of the state written
 };
 
 // Arguments of the initialisation kernel.
@@ -161,11 +161,13 @@ cudaError_t launch_aa(const StepArgs& a, int kind, int storage, bool odd, bool m
 cudaError_t launch_aa_init(const StepArgs& a, int kind, int storage, const float* rho, const float* u,
                            const float* theta, cudaStream_t s);
 
-// Wall-bounded D2Q37 step (walls.cu), in launch order: mode 2 = the FP64
-// completion of the wall rows' unknowns into a.comp, mode 0 = the moments
-// launch (moments into mcur / the readout pointers, partials), mode 1 = the
-// collide launch (thermal: with H_i).  Modes 0 and 1 read a.comp.
-cudaError_t launch_walls(const WallArgs& a, int storage, int mode, bool thermal, cudaStream_t s);
+// Wall-bounded D2Q37 (walls.cu).  A step is LOWER, UPPER and BETWEEN, in any
+// order or at once (thermal: with H_i): they read a.fin and a.comp and write
+// a.fout, a.mcur and a.comp_next.  COMPLETE fills a.comp_next from a.fin and
+// a.mprev; MOMENTS is the readout (the readout pointers, partials) of a.fin and
+// a.comp.
+enum WallLaunch { WALL_LOWER, WALL_UPPER, WALL_BETWEEN, WALL_COMPLETE, WALL_MOMENTS };
+cudaError_t launch_walls(const WallArgs& a, int storage, WallLaunch what, bool thermal, cudaStream_t s);
 // Initial state of a wall-bounded context into a.fout and m [4][N] = rho,
 // u_x, u_y, theta - 1 of the initial fields.
 cudaError_t launch_wall_init(const WallArgs& a, int storage, const float* rho, const float* u, const float* theta,

@@ -32,15 +32,14 @@
 // (h* = (1 - omega) h + omega (g^eq - r) + beta S), and the completion is
 // the same in h as in g (r_i = r_ibar).
 //
-// Each step is three launches: wall_complete_kernel completes the unknowns of
-// the six wall rows in FP64 into a small buffer; wall_moments_kernel pulls
-// every node's populations (the unknowns from that buffer) and writes its
-// moments (rho, u, theta - 1) of time t, which are the next step's targets and
-// the neighbour temperatures of grad theta; wall_collide_kernel pulls again,
-// collides (Eq. 4.4 with F_i and H_i) and stores.  grad theta is a
-// second-order central difference, one-sided into the fluid at the wall rows.
-// Two reads of the populations per step: these domains are the paper's
-// validation cases, a few thousand to a few hundred thousand nodes.
+// Each step is three launches that run beside one another: the kEdge rows next
+// to the lower and to the upper wall (wall_edge_kernel, which also completes
+// the unknowns of the state that it writes, in FP64, for the next step) and the
+// rows between (wall_step_kernel).  Each pulls the populations once (the
+// unknowns from the completion buffer), forms the moments (rho, u, theta - 1)
+// of time t, grad theta (second-order central differences, one-sided into the
+// fluid at the wall rows) from them, collides (Eq. 4.4 with F_i and H_i) and
+// stores.
 #include "internal.h"
 #include "lattice.cuh"
 #include "step_common.cuh"
@@ -53,70 +52,51 @@ namespace {
 using L = D2Q37;
 constexpr int kBX = 32, kBY = 8;
 
-__host__ __device__ constexpr int opp_of(int i) { return i == 0 ? 0 : (((i - 1) & 1) ? i - 1 : i + 1); }
-
 __device__ __forceinline__ int wrapx(int v, int n) {
   return v < 0 ? v + n : (v >= n ? v - n : v);
 }
 
-// P_i - 1 for f^eq_i = w_i rho P_i (Eq. 2.2): the Hermite expansion
-// sum_{a+b<=4} m_a(u_x) m_b(u_y) He_a(xi_x) He_b(xi_y) / (a! b!), without the
-// (0, 0) term, u in units of c0, m_a the Hermite moments of a Gaussian of
-// variance 1 + tb.  FP64: the completion differences two such values whose
+// Hermite moments m_0..m_4 of a Gaussian of mean u (in units of c0) and
+// variance 1 + tb.  FP64: the completion differences two equilibria whose
 // difference is O(u), which FP32 would leave with O(1e-7) absolute error at
 // every wall node and step (a drift in mass and momentum at the walls).
 __device__ __forceinline__ void gauss_moments_d(double u, double tb, double (&m)[5]) {
-  const double u2 = u * u;
+  const double u2 = __dmul_rn(u, u);
   m[0] = 1.0;
   m[1] = u;
-  m[2] = u2 + tb;
-  m[3] = u * (u2 + 3.0 * tb);
-  m[4] = u2 * (u2 + 6.0 * tb) + 3.0 * tb * tb;
+  m[2] = __dadd_rn(u2, tb);
+  m[3] = __dmul_rn(u, fma(3.0, tb, u2));
+  m[4] = fma(u2, fma(6.0, tb, u2), __dmul_rn(3.0, __dmul_rn(tb, tb)));
 }
-// P_i - 1 from precomputed products: hp[k] = m_a(u_x) m_b(u_y) for
-// the 14 index pairs (a, b) with 1 <= a + b <= 4 (k = hk(a, b)), so that the
-// completion forms the products once per state (the node's previous moments,
-// and one wall target per |c_y|) and then costs 14 FP64 multiply-adds per
-// population instead of a whole expansion.
-__host__ __device__ constexpr int hk(int a, int b) {
-  return (a + b == 1) ? a : (a + b == 2) ? 2 + a : (a + b == 3) ? 5 + a : 9 + a;
+// He_a(c / c0) / a! at an integer c
+__host__ __device__ constexpr double hea(int a, int c) {
+  double s = 0.0;
+  for (int p = 0; p <= a; ++p) s += he(a, p) * ipow_d((double)c / L::c0, p);
+  return s / fact_d(a);
 }
-__device__ __forceinline__ void herm_prod(double ux, double uy, double tb, double (&hp)[14]) {
-  double mx[5], my[5];
-  gauss_moments_d(ux * (1.0 / L::c0), tb, mx);
-  gauss_moments_d(uy * (1.0 / L::c0), tb, my);
-  static_for<5>([&](auto A) {
-    static_for<5>([&](auto B) {
-      constexpr int a = A, b = B;
-      if constexpr (a + b >= 1 && a + b <= L::FEQ_ORDER) hp[hk(a, b)] = mx[a] * my[b];
-    });
-  });
+// index of the velocity (cx, cy), -1 if the lattice has none
+__host__ __device__ constexpr int vel_index(int cx, int cy) {
+  for (int i = 0; i < L::Q; ++i)
+    if (L::c(i, 0) == cx && L::c(i, 1) == cy) return i;
+  return -1;
 }
-template <int I>
-__device__ __forceinline__ double peq_m1_hp(const double (&hp)[14]) {
-  constexpr int cx = L::c(I, 0), cy = L::c(I, 1);
-  double acc = 0.0;
-  static_for<5>([&](auto A) {
-    static_for<5>([&](auto B) {
-      constexpr int a = A, b = B;
-      if constexpr (a + b >= 1 && a + b <= L::FEQ_ORDER) {
-        constexpr double hx = [] {
-          double s = 0.0;
-          for (int p = 0; p <= a; ++p) s += he(a, p) * ipow_d((double)cx / L::c0, p);
-          return s;
-        }();
-        constexpr double hy = [] {
-          double s = 0.0;
-          for (int q = 0; q <= b; ++q) s += he(b, q) * ipow_d((double)cy / L::c0, q);
-          return s;
-        }();
-        constexpr double cf = hx * hy / (fact_d(a) * fact_d(b));
-        if constexpr (cf != 0.0) acc = fma(cf, hp[hk(a, b)], acc);
-      }
-    });
-  });
-  return acc;
+template <int CX, int CY>
+constexpr int kVel = vel_index(CX, CY);
+template <int A, int C>
+constexpr double kHea = hea(A, C);
+// one of three compile-time values by k = 1, 2, 3
+template <class T>
+__device__ __forceinline__ T pick3(int k, T a, T b, T c) {
+  return k == 1 ? a : (k == 2 ? b : c);
 }
+// sum over the velocities (cx, k) of w (ORD 0) or w He_ORD(c_x / c0) / ORD!
+template <int K, int ORD>
+constexpr double kRowSum = [] {
+  double s = 0.0;
+  for (int cx = -3; cx <= 3; ++cx)
+    if (vel_index(cx, K) >= 0) s += L::w(vel_index(cx, K)) * (ORD ? hea(ORD, cx) : 1.0);
+  return s;
+}();
 
 template <int ST>
 __device__ __forceinline__ float ldpop(const WallArgs& a, int i, int x, int y) {
@@ -139,68 +119,190 @@ __device__ __forceinline__ void wall_accel(const WallArgs& a, int node, int y, f
   }
 }
 
-// Completion of the unknowns of a wall-row node (x, y), r = 0, 1, 2 rows from
-// its wall node: written to a.comp[slot][i][x] (slot = 3 side + r) for every
-// unknown i.  It runs once per step, before the two launches that read the
-// populations, in a launch of its own over the six wall rows, so that its
-// FP64 arithmetic neither stalls the blocks of the full-domain launches nor
-// is done twice.
-template <int ST>
-__device__ __forceinline__ void wall_complete(const WallArgs& a, int x, int y) {
-  const int nx = a.nx, ny = a.ny;
-  const int side = (y < ny / 2) ? 0 : 1;
-  const int r = side == 0 ? y : ny - 1 - y;
-  const size_t N = (size_t)a.N;
-  const int node = y * nx + x;
-  const int node1 = (side == 0 ? 1 : ny - 2) * nx + x;
-  const double rp = __ldg(a.mprev + node);
-  const double upx = __ldg(a.mprev + N + node), upy = __ldg(a.mprev + 2 * N + node);
-  const double tbp = __ldg(a.mprev + 3 * N + node);
-  const double u1x = __ldg(a.mprev + N + node1), u1y = __ldg(a.mprev + 2 * N + node1);
-  const double tb1 = __ldg(a.mprev + 3 * N + node1);
-  const double uwx = a.wall_u[side][0], uwy = a.wall_u[side][1], tbw = a.wall_tb[side];
-  // Hermite products of the previous moments and of the wall target of each
-  // |c_y| = 1, 2, 3 (extrapolated to the turning point)
-  double hpp[14], hpt[3][14];
-  herm_prod(upx, upy, tbp, hpp);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const double wgt = (double)(2 + k - 2 * r);   // (1/2 - turning point) / (1/2), |c_y| = k + 1
-    herm_prod(fma(wgt, uwx - u1x, uwx), fma(wgt, uwy - u1y, uwy), fma(wgt, tbw - tb1, tbw), hpt[k]);
+// Completion of the unknowns of the wall rows r = 0, 1, 2 of one wall: those
+// with |c_y| > r that point into the fluid.
+//
+// One lane takes the velocities (cx, k), cx = -3..3, of one row |c_y| = k of
+// one node, so a column has six tasks (r, k > r), lanes 6 c + t for the c-th of
+// a warp's kCols columns.  With the prefix sums T_n = sum_{1 <= b <= n} He_b(k /
+// c0) / b! m_b(u_y), P(c) = f^eq_c / (w_c rho) truncated at a + b <= 4 is
+//   P - 1 = T_4 + sum_{a = 1..4} He_a(c_x / c0) / a! R_a,  R_a = m_a(u_x) (1 + T_{4-a}),
+// and the bracket of the completion, with t the target and p the previous state,
+//   s P_t - P_p = T' + sum_a He_a(c_x / c0) / a! R'_a,
+//   T' = (s - 1) + (s - 1) T_4,t + (T_4,t - T_4,p),  R'_a = (s - 1) R_a,t + (R_a,t - R_a,p),
+// whose even and odd halves +c_x and -c_x share.  s is a sum over the rows k
+// of a node, exchanged by shuffles.
+//
+// A warp's FP64 instruction holds its quarter of the SM for 64 clocks here
+// (measured, with one active lane as with 32, and dependent or not), so the
+// chain of FP64 instructions of a warp is what the completion takes, and four
+// warps on the four quarters run it four times as fast as one: the warps take
+// the x and the y moments of the target and of the previous state, then the
+// differences beside the scale's division, then one |c_x| each.  The longest
+// chain is 53 instructions.  A step of 200 x 102 takes 7.4 us with it, 11.1 us
+// with all 170 instructions in one warp, and took 49 us (47 us of them the
+// completion) with one thread per node and a whole expansion per population.
+constexpr int kCols = 4;    // columns of a block
+constexpr int kCompWarps = 4;
+
+// moments of a node of the previous step and its column's first fluid row, and
+// the populations that left, of the rows 0 .. 2 of a block (index r kCols + column)
+struct CompIn {
+  float mom[3 * kCols][4];       // rho, u_x, u_y, theta - 1
+  float post[37][3 * kCols];     // the state as stored
+};
+struct CompShared {
+  double v[24][32];              // values that the four warps exchange, per lane
+};
+
+__device__ __forceinline__ void comp_barrier() { asm volatile("barrier.sync 2, 128;" ::: "memory"); }
+
+// Called by four whole warps (wq = 0 .. 3); moments_ready() and state_ready()
+// return once in.mom and in.post are written.  x0: first column of the block.
+template <class M, class P>
+__device__ __forceinline__ void complete_columns(const WallArgs& a, int side, int x0, int wq, int lane, const CompIn& in,
+                                                 CompShared& sh, M&& moments_ready, P&& state_ready) {
+  const int lc = lane / 6, t = lane - 6 * lc;
+  const int col = lc < kCols ? lc : kCols - 1;          // lanes past the last column repeat it
+  const int r = t < 3 ? 0 : (t < 5 ? 1 : 2);            // rows from the wall node
+  const int k = t < 3 ? t + 1 : (t < 5 ? t - 1 : 3);    // |c_y|
+  int first = 6 * lc + (r == 0 ? 0 : (r == 1 ? 3 : 5)); // lane of the node's first task
+  if (lc >= kCols) first = 0;
+  enum { TT = 0, TP = 4, RT = 8, AT = 12, RP = 13, BP = 17, SM1 = 18, TPR = 19, RPR = 20 };
+  const double hb1 = pick3(k, kHea<1, 1>, kHea<1, 2>, kHea<1, 3>), hb2 = pick3(k, kHea<2, 1>, kHea<2, 2>, kHea<2, 3>);
+  const double hb3 = pick3(k, kHea<3, 1>, kHea<3, 2>, kHea<3, 3>), hb4 = pick3(k, kHea<4, 1>, kHea<4, 2>, kHea<4, 3>);
+  // sums over a row's velocities of w and of w He_2 / 2!, w He_4 / 4! (the odd halves cancel)
+  const double w0 = pick3(k, kRowSum<1, 0>, kRowSum<2, 0>, kRowSum<3, 0>);
+  const double w2 = pick3(k, kRowSum<1, 2>, kRowSum<2, 2>, kRowSum<3, 2>);
+  const double w4 = pick3(k, kRowSum<1, 4>, kRowSum<2, 4>, kRowSum<3, 4>);
+  moments_ready();
+  // phase 1: the Gaussian moments of one component of one state.  P(c; u) is
+  // even in (c, u) per axis, so the rows are evaluated at c_y = +k, with u_y
+  // mirrored at the upper wall, and the previous state, taken at the opposite
+  // velocity, with -u.
+  const float* p = in.mom[r * kCols + col];
+  double m[5];
+  {
+    const bool yax = wq & 1;
+    double u, tb;
+    if (wq < 2) {   // the wall target at the turning point, extrapolated through the first fluid row
+      const float* q = in.mom[kCols + col];
+      const double wgt = (double)(1 + k - 2 * r);       // (1/2 - turning point) / (1/2)
+      const double uw = a.wall_u[side][yax], tw = a.wall_tb[side];
+      u = fma(wgt, __dsub_rn(uw, (double)(yax ? q[2] : q[1])), uw);
+      if (yax && side) u = -u;
+      tb = fma(wgt, __dsub_rn(tw, (double)q[3]), tw);
+    } else {
+      const float v = yax ? p[2] : p[1];
+      u = (double)((yax && side) ? v : -v);
+      tb = (double)p[3];
+    }
+    gauss_moments_d(__dmul_rn(u, 1.0 / L::c0), tb, m);
+    if (yax) {
+      double T = __dmul_rn(hb1, m[1]);
+      const int o = wq == 1 ? TT : TP;
+      sh.v[o][lane] = T;
+      sh.v[o + 1][lane] = T = fma(hb2, m[2], T);
+      sh.v[o + 2][lane] = T = fma(hb3, m[3], T);
+      sh.v[o + 3][lane] = fma(hb4, m[4], T);
+    }
   }
-  // sums over the unknowns of w P_i(targets) - w and w P_ibar(p) - w
-  double W = 0.0, A = 0.0, B = 0.0;
-  static_for<37>([&](auto I) {
-    constexpr int i = I;
-    constexpr int cy = L::c(i, 1), ab = cy < 0 ? -cy : cy;
-    constexpr int b = opp_of(i);
-    if constexpr (ab > 0) {
-      if (y - cy < 0 || y - cy >= ny) {
-        constexpr double w = L::w(i);
-        W += w;
-        A = fma(w, peq_m1_hp<i>(hpt[ab - 1]), A);
-        B = fma(w, peq_m1_hp<b>(hpp), B);
-      }
+  comp_barrier();
+  // phase 2: R_a of each state, and the sums over the row's velocities of w (P - 1)
+  if (!(wq & 1)) {
+    const int o = wq == 0 ? TT : TP, d = wq == 0 ? RT : RP;
+    const double r2 = fma(m[2], sh.v[o + 1][lane], m[2]);
+    sh.v[d][lane] = fma(m[1], sh.v[o + 2][lane], m[1]);
+    sh.v[d + 1][lane] = r2;
+    sh.v[d + 2][lane] = fma(m[3], sh.v[o][lane], m[3]);
+    sh.v[d + 3][lane] = m[4];
+    sh.v[d + 4][lane] = fma(w4, m[4], fma(w2, r2, __dmul_rn(w0, sh.v[o + 3][lane])));
+  }
+  comp_barrier();
+  // phase 3: s - 1 = sum_rows (B - A) / sum_rows (W + A), and beside it the differences
+  double x1 = 0.0, d1 = 0.0, x2 = 0.0, d2 = 0.0;
+  if (wq == 3) {
+    const double A = sh.v[AT][lane], B = sh.v[BP][lane];
+    const double d = __dsub_rn(B, A), sw = __dadd_rn(w0, A);
+    double D = 0.0, S = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int src = first + (j < 3 - r ? j : 0);
+      const double dj = __shfl_sync(0xffffffffu, d, src), sj = __shfl_sync(0xffffffffu, sw, src);
+      D = j == 0 ? dj : (j < 3 - r ? __dadd_rn(D, dj) : D);
+      S = j == 0 ? sj : (j < 3 - r ? __dadd_rn(S, sj) : S);
     }
-  });
-  const double sm1 = (B - A) / (W + A);            // s - 1
-  float* comp = a.comp + (size_t)(3 * side + r) * 37 * nx + x;
-  static_for<37>([&](auto I) {
-    constexpr int i = I;
-    constexpr int cy = L::c(i, 1), ab = cy < 0 ? -cy : cy;
-    constexpr int b = opp_of(i);
-    if constexpr (ab > 0) {
-      if (y - cy < 0 || y - cy >= ny) {
-        const double pi = peq_m1_hp<i>(hpt[ab - 1]), pb = peq_m1_hp<b>(hpp);
-        // s P_i - P_ibar = (s - 1) + s (P_i - 1) - (P_ibar - 1)
-        comp[(size_t)i * nx] = (float)fma(rp, sm1 + fma(sm1, pi, pi) - pb, (double)ldpop<ST>(a, b, x, y));
-      }
+    sh.v[SM1][lane] = D / S;
+  } else if (wq == 0) {
+    x1 = sh.v[TT + 3][lane];
+    d1 = __dsub_rn(x1, sh.v[TP + 3][lane]);
+  } else {
+    const int i = wq - 1;   // R_1, R_3 or R_2, R_4
+    x1 = sh.v[RT + i][lane];
+    d1 = __dsub_rn(x1, sh.v[RP + i][lane]);
+    x2 = sh.v[RT + i + 2][lane];
+    d2 = __dsub_rn(x2, sh.v[RP + i + 2][lane]);
+  }
+  comp_barrier();
+  // phase 4: T' and R'_a
+  if (wq != 3) {
+    const double sm1 = sh.v[SM1][lane];
+    if (wq == 0) {
+      sh.v[TPR][lane] = __dadd_rn(sm1, fma(sm1, x1, d1));
+    } else {
+      sh.v[RPR + wq - 1][lane] = fma(sm1, x1, d1);
+      sh.v[RPR + wq + 1][lane] = fma(sm1, x2, d2);
     }
-  });
+  }
+  comp_barrier();
+  const double rp = p[0];
+  state_ready();
+  // phase 5: the velocities (+-cx, k), cx = wq: g_i = g*_ibar + rho_p (s P_i - P_ibar)
+  const int x = x0 + col;
+  if (lane < 6 * kCols && x < a.nx) {
+    float* out = a.comp_next + (size_t)(3 * side + r) * 37 * a.nx + x;
+    const int at = r * kCols + col;
+    static_for<4>([&](auto Cx) {
+      constexpr int cx = Cx;
+      if (wq == cx) {
+        constexpr double h1 = kHea<1, cx>, h2 = kHea<2, cx>, h3 = kHea<3, cx>, h4 = kHea<4, cx>;
+        const double E = fma(h4, sh.v[RPR + 3][lane], fma(h2, sh.v[RPR + 1][lane], sh.v[TPR][lane]));
+        const double O = cx == 0 ? 0.0 : fma(h3, sh.v[RPR + 2][lane], __dmul_rn(h1, sh.v[RPR][lane]));
+        static_for<(cx == 0 ? 1 : 2)>([&](auto Sg) {
+          constexpr int c = Sg == 0 ? cx : -cx;
+          const int up = pick3(k, kVel<c, 1>, kVel<c, 2>, kVel<c, 3>), dn = pick3(k, kVel<c, -1>, kVel<c, -2>, kVel<c, -3>);
+          const int bu = pick3(k, kVel<-c, -1>, kVel<-c, -2>, kVel<-c, -3>);
+          const int bd = pick3(k, kVel<-c, 1>, kVel<-c, 2>, kVel<-c, 3>);
+          const double br = cx == 0 ? E : (Sg == 0 ? __dadd_rn(E, O) : __dsub_rn(E, O));
+          if (up >= 0)
+            out[(size_t)(side == 0 ? up : dn) * a.nx] = (float)fma(rp, br, (double)in.post[side == 0 ? bu : bd][at]);
+        });
+      }
+    });
+  }
+}
+
+// The completion from a stored state and its moments (after hlbm_init and
+// hlbm_load; a step completes the state that it writes itself): blockIdx.y the
+// wall.
+template <int ST>
+__global__ void __launch_bounds__(32 * kCompWarps) wall_complete_kernel(const __grid_constant__ WallArgs a) {
+  __shared__ CompIn in;
+  __shared__ CompShared sh;
+  const int side = blockIdx.y, x0 = blockIdx.x * kCols;
+  const size_t N = (size_t)a.N;
+  for (int q = threadIdx.x; q < 41 * 3 * kCols; q += blockDim.x) {
+    const int i = q / (3 * kCols), at = q - i * 3 * kCols, r = at / kCols;
+    const int y = side == 0 ? r : a.ny - 1 - r, x = min(x0 + at - r * kCols, a.nx - 1);
+    if (i < 37) in.post[i][at] = ldpop<ST>(a, i, x, y);
+    else in.mom[at][i - 37] = __ldg(a.mprev + (size_t)(i - 37) * N + y * a.nx + x);
+  }
+  __syncthreads();
+  complete_columns(a, side, x0, threadIdx.x >> 5, threadIdx.x & 31, in, sh, [] {}, [] {});
 }
 
 // The 37 populations of node (x, y) at time t after streaming, the unknowns
-// at the walls taken from the completion launch.
+// at the walls taken from the completion buffer.
 template <int ST>
 __device__ __forceinline__ void wall_gather(const WallArgs& a, int x, int y, float (&g)[37]) {
   const int nx = a.nx, ny = a.ny;
@@ -319,12 +421,6 @@ __global__ void __launch_bounds__(kBX * kBY, 4) wall_moments_kernel(const __grid
     const int node = y * a.nx + x;
     const WallMoments m = wall_moments(a, g, node, y);
     const size_t N = (size_t)a.N;
-    if (a.mcur) {
-      a.mcur[node] = m.rho;
-      a.mcur[N + node] = m.ux;
-      a.mcur[2 * N + node] = m.uy;
-      a.mcur[3 * N + node] = m.tb;
-    }
     if (a.rho_out) a.rho_out[node] = m.rho;
     if (a.u_out) {
       a.u_out[node] = m.ux;
@@ -357,28 +453,13 @@ __global__ void __launch_bounds__(kBX * kBY, 4) wall_moments_kernel(const __grid
   }
 }
 
-template <int ST, bool THERMAL>
-__global__ void __launch_bounds__(kBX * kBY, 3) wall_collide_kernel(const __grid_constant__ WallArgs a) {
-  const int x = blockIdx.x * kBX + threadIdx.x, y = blockIdx.y * kBY + threadIdx.y;
-  if (x >= a.nx || y >= a.ny) return;
-  const int nx = a.nx, ny = a.ny;
-  const size_t N = (size_t)a.N;
-  const int node = y * nx + x;
-  float g[37];
-  wall_gather<ST>(a, x, y, g);
-  const WallMoments m = wall_moments(a, g, node, y);
+// grad theta's term and the collision of one node: g (the local deviations of
+// wall_moments) becomes the post-collision state
+template <bool THERMAL>
+__device__ __forceinline__ void wall_collide(const WallArgs& a, const WallMoments& m, float gtx, float gty, float (&g)[37]) {
   NodeSrcT<float> s;
   s.hG[0] = s.hG[1] = s.hG[2] = 0.f;
   if constexpr (THERMAL) {
-    const float* tb = a.mcur + 3 * N;
-    const float gtx = 0.5f * (tb[y * nx + wrapx(x + 1, nx)] - tb[y * nx + wrapx(x - 1, nx)]);
-    float gty;
-    if (y == 0)
-      gty = 0.5f * (-3.f * tb[node] + 4.f * tb[node + nx] - tb[node + 2 * nx]);
-    else if (y == ny - 1)
-      gty = -0.5f * (-3.f * tb[node] + 4.f * tb[node - nx] - tb[node - 2 * nx]);
-    else
-      gty = 0.5f * (tb[node + nx] - tb[node - nx]);
     // s^(3) += rho theta (1 - 1/Pr) [delta grad_xi theta], grad_xi = c0 grad
     const float hc = m.rho * (1.f + m.tb) * (a.h_coef * (float)L::c0);
     s.hG[0] = hc * gtx;
@@ -400,13 +481,180 @@ __global__ void __launch_bounds__(kBX * kBY, 3) wall_collide_kernel(const __grid
   const float om1 = 1.f - a.omega;
   K[0] = fmaf(-om1, m.acc, K[0]);
   apply_poly_h<L, 15>(g, K, om1, m.dr);
+}
+
+__device__ __forceinline__ void store_moments(const WallArgs& a, const WallMoments& m, int node) {
+  const size_t N = (size_t)a.N;
+  a.mcur[node] = m.rho;
+  a.mcur[N + node] = m.ux;
+  a.mcur[2 * N + node] = m.uy;
+  a.mcur[3 * N + node] = m.tb;
+}
+
+// The step of the kEdge rows next to one wall, and the completion of the state
+// it writes.  A block owns kCols columns.  Its first warp takes the 16 nodes
+// and, with H_i, the ring of 12 around them for theta; given their moments,
+// its other four warps form the completion's brackets in FP64 while the first
+// collides, and complete the unknowns of rows 0 .. 2 from the new state.  So
+// no launch of a step waits for another one, and the FP64 work is spread over
+// nx / 2 blocks.
+constexpr int kEdge = 4;
+constexpr int kEdgeThreads = 32 * (1 + kCompWarps);
+
+// the block's barrier, from the different code of its warps
+__device__ __forceinline__ void edge_barrier() { asm volatile("barrier.sync 1, 160;" ::: "memory"); }
+
+template <int ST, bool THERMAL>
+__global__ void __launch_bounds__(kEdgeThreads) wall_edge_kernel(const __grid_constant__ WallArgs a, int side) {
+  constexpr int TW = kCols + 2;
+  __shared__ float tbs[(kEdge + 1) * TW];       // theta - 1 by rows from the wall, columns x0 - 1 .. x0 + kCols
+  __shared__ CompIn in;
+  __shared__ CompShared sh;
+  using T = typename Codec<ST>::T;
+  const int nx = a.nx, ny = a.ny;
+  const size_t N = (size_t)a.N;
+  const int lane = threadIdx.x & 31, x0 = blockIdx.x * kCols;
+  if (threadIdx.x < 32) {
+    // lanes 0 .. 15 the nodes, 16 .. 19 row kEdge, 20 .. 23 and 24 .. 27 the
+    // columns to the left and right
+    int r, c;
+    if (lane < kEdge * kCols) {
+      r = lane / kCols;
+      c = lane - r * kCols;
+    } else if (lane < kEdge * kCols + kCols) {
+      r = kEdge;
+      c = lane - kEdge * kCols;
+    } else {
+      const int q = lane - (kEdge + 1) * kCols;
+      r = q & (kEdge - 1);
+      c = q < kEdge ? -1 : kCols;
+    }
+    const int y = side == 0 ? r : ny - 1 - r;
+    int x = x0 + c;
+    // a domain of fewer than 2 kEdge rows: the lower wall's block stores the rows up to kEdge - 1
+    const bool store = lane < kEdge * kCols && x < nx && (side == 0 || y >= kEdge);
+    // column nx is column 0, the right neighbour of the last one
+    const bool needed = lane < (kEdge + 1) * kCols + 2 * kEdge && (store || (THERMAL && x <= nx));
+    if (x < 0) x += nx;
+    else if (x >= nx) x -= nx;
+    const int node = y * nx + x;
+    float g[37];
+    WallMoments m;
+    if (needed) {
+      wall_gather<ST>(a, x, y, g);
+      m = wall_moments(a, g, node, y);
+      if constexpr (THERMAL) tbs[r * TW + c + 1] = m.tb;
+      if (lane < 3 * kCols) {
+        in.mom[lane][0] = m.rho;
+        in.mom[lane][1] = m.ux;
+        in.mom[lane][2] = m.uy;
+        in.mom[lane][3] = m.tb;
+      }
+    }
+    edge_barrier();
+    if (store) {
+      float gtx = 0.f, gty = 0.f;
+      if constexpr (THERMAL) {
+        const float* tb = tbs + r * TW + c + 1;
+        gtx = 0.5f * (tb[1] - tb[-1]);
+        if (r == 0) {
+          gty = (side == 0 ? 0.5f : -0.5f) * (-3.f * tb[0] + 4.f * tb[TW] - tb[2 * TW]);
+        } else {
+          gty = side == 0 ? 0.5f * (tb[TW] - tb[-TW]) : 0.5f * (tb[-TW] - tb[TW]);
+        }
+      }
+      wall_collide<THERMAL>(a, m, gtx, gty, g);
+      store_moments(a, m, node);
+      const uint32_t salt = std::is_same<T, float>::value ? 0u : node_salt(node, g[0]);
+      if (HLBM_IN(node, a.N, DBG_STORE)) {
+        T* __restrict__ fout = static_cast<T*>(a.fout) + node;
+        static_for<37>([&](auto I) {
+          constexpr int i = I;
+          const T v = round_store<T>(g[i], pop_bits(salt, i));
+          fout[(size_t)i * N] = v;
+          if (lane < 3 * kCols) in.post[i][lane] = to_float(v);
+        });
+      }
+    }
+    edge_barrier();
+  } else {
+    complete_columns(a, side, x0, (threadIdx.x >> 5) - 1, lane, in, sh, [] { edge_barrier(); }, [] { edge_barrier(); });
+  }
+}
+
+// The step of the rows kEdge .. ny - 1 - kEdge, whose pulls and ring cross no
+// wall: moments, grad theta and collision in one pass.  A block owns kBX x kBY
+// nodes, one thread each, whose populations stay in registers; with H_i, three
+// more warps pull the 80 nodes of the 4-neighbour ring around them for theta
+// alone (their lines are the neighbour blocks', in L1 or L2), so the
+// populations are read from memory once per step (two passes, a moments launch
+// and a collide launch, took 33 + 57 us at 1024 x 1026; this one takes 72 us).
+template <bool THERMAL>
+constexpr int wall_threads() {
+  return kBX * kBY + (THERMAL ? 96 : 0);
+}
+
+template <int ST, bool THERMAL>
+__global__ void __launch_bounds__(wall_threads<THERMAL>(), THERMAL ? 2 : 3)
+    wall_step_kernel(const __grid_constant__ WallArgs a) {
+  constexpr int SW = kBX + 2, RING = 2 * kBX + 2 * kBY;
+  __shared__ float tbs[THERMAL ? (kBY + 2) * SW : 1];   // theta - 1 of the block and its ring
+  const int nx = a.nx, yhi = a.ny - kEdge;
+  const size_t N = (size_t)a.N;
+  const int tid = threadIdx.x;
+  const int x0 = blockIdx.x * kBX, y0 = kEdge + kBY * (int)blockIdx.y;
+  // region coordinates (0 .. kBX + 1, 0 .. kBY + 1) of this thread's node
+  int i, j;
+  if (tid < kBX * kBY) {
+    i = (tid & (kBX - 1)) + 1;
+    j = tid / kBX + 1;
+  } else {
+    const int q = tid - kBX * kBY;
+    if (q >= RING) i = j = -1;
+    else if (q < 2 * kBX) {
+      i = (q & (kBX - 1)) + 1;
+      j = q < kBX ? 0 : kBY + 1;
+    } else {
+      const int p = q - 2 * kBX;
+      i = p < kBY ? 0 : kBX + 1;
+      j = (p & (kBY - 1)) + 1;
+    }
+  }
+  const int y = y0 + j - 1;
+  int x = x0 + i - 1;
+  const bool store = tid < kBX * kBY && x < nx && y < yhi;
+  // column nx is column 0, the right neighbour of the last one; rows past yhi are not touched
+  const bool needed = j >= 0 && y <= yhi && (store || (THERMAL && x <= nx));
+  if (x < 0) x += nx;
+  else if (x >= nx) x -= nx;
+  const int node = y * nx + x;
+  float g[37];
+  WallMoments m;
+  if (needed) {
+    static_for<37>([&](auto I) {
+      constexpr int q = I;
+      g[q] = ldpop<ST>(a, q, wrapx(x - L::c(q, 0), nx), y - L::c(q, 1));
+    });
+    m = wall_moments(a, g, node, y);
+    if constexpr (THERMAL) tbs[j * SW + i] = m.tb;
+  }
+  if constexpr (THERMAL) __syncthreads();
+  if (!store) return;
+  store_moments(a, m, node);
+  float gtx = 0.f, gty = 0.f;
+  if constexpr (THERMAL) {
+    const float* tb = tbs + j * SW + i;
+    gtx = 0.5f * (tb[1] - tb[-1]);
+    gty = 0.5f * (tb[SW] - tb[-SW]);
+  }
+  wall_collide<THERMAL>(a, m, gtx, gty, g);
   using T = typename Codec<ST>::T;
   if (!HLBM_IN(node, a.N, DBG_STORE)) return;
   T* __restrict__ fout = static_cast<T*>(a.fout) + node;
   const uint32_t salt = std::is_same<T, float>::value ? 0u : node_salt(node, g[0]);
   static_for<37>([&](auto I) {
-    constexpr int i = I;
-    fout[(size_t)i * N] = round_store<T>(g[i], pop_bits(salt, i));
+    constexpr int q = I;
+    fout[(size_t)q * N] = round_store<T>(g[q], pop_bits(salt, q));
   });
 }
 
@@ -452,32 +700,29 @@ __global__ void __launch_bounds__(256) wall_init_kernel(const __grid_constant__ 
   });
 }
 
-// One thread per node of the six wall rows (rows 0, 1, 2 and ny - 1, ny - 2,
-// ny - 3), one warp per block so that the FP64 work spreads over the SMs.
-template <int ST>
-__global__ void __launch_bounds__(32) wall_complete_kernel(const __grid_constant__ WallArgs a) {
-  const int t = blockIdx.x * 32 + threadIdx.x;
-  if (t >= 6 * a.nx) return;
-  const int slot = t / a.nx, x = t - slot * a.nx;
-  const int y = slot < 3 ? slot : a.ny - 1 - (slot - 3);
-  wall_complete<ST>(a, x, y);
+template <int ST, bool THERMAL>
+cudaError_t launch_wall_step(const WallArgs& a, WallLaunch what, cudaStream_t s) {
+  if (what == WALL_BETWEEN) {
+    if (a.ny <= 2 * kEdge) return cudaSuccess;
+    const dim3 grid((a.nx + kBX - 1) / kBX, (a.ny - 2 * kEdge + kBY - 1) / kBY);
+    wall_step_kernel<ST, THERMAL><<<grid, wall_threads<THERMAL>(), 0, s>>>(a);
+  } else {
+    wall_edge_kernel<ST, THERMAL><<<(a.nx + kCols - 1) / kCols, kEdgeThreads, 0, s>>>(a, what == WALL_UPPER ? 1 : 0);
+  }
+  return cudaGetLastError();
 }
 
 template <int ST>
-cudaError_t launch_walls_st(const WallArgs& a, int mode, bool thermal, cudaStream_t s) {
-  if (mode == 2) {
-    wall_complete_kernel<ST><<<(6 * a.nx + 31) / 32, 32, 0, s>>>(a);
+cudaError_t launch_walls_st(const WallArgs& a, WallLaunch what, bool thermal, cudaStream_t s) {
+  if (what == WALL_COMPLETE) {
+    wall_complete_kernel<ST><<<dim3((a.nx + kCols - 1) / kCols, 2), 32 * kCompWarps, 0, s>>>(a);
     return cudaGetLastError();
   }
-  const bool collide = mode == 1;
-  const dim3 block(kBX, kBY), grid((a.nx + kBX - 1) / kBX, (a.ny + kBY - 1) / kBY);
-  if (!collide)
-    wall_moments_kernel<ST><<<grid, block, 0, s>>>(a);
-  else if (thermal)
-    wall_collide_kernel<ST, true><<<grid, block, 0, s>>>(a);
-  else
-    wall_collide_kernel<ST, false><<<grid, block, 0, s>>>(a);
-  return cudaGetLastError();
+  if (what == WALL_MOMENTS) {
+    wall_moments_kernel<ST><<<dim3((a.nx + kBX - 1) / kBX, (a.ny + kBY - 1) / kBY), dim3(kBX, kBY), 0, s>>>(a);
+    return cudaGetLastError();
+  }
+  return thermal ? launch_wall_step<ST, true>(a, what, s) : launch_wall_step<ST, false>(a, what, s);
 }
 
 }  // namespace
@@ -493,11 +738,11 @@ cudaError_t launch_wall_init(const WallArgs& a, int storage, const float* rho, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_walls(const WallArgs& a, int storage, int mode, bool thermal, cudaStream_t s) {
+cudaError_t launch_walls(const WallArgs& a, int storage, WallLaunch what, bool thermal, cudaStream_t s) {
   switch (storage) {
-    case ST_F32: return launch_walls_st<ST_F32>(a, mode, thermal, s);
-    case ST_F16: return launch_walls_st<ST_F16>(a, mode, thermal, s);
-    default: return launch_walls_st<ST_BF16>(a, mode, thermal, s);
+    case ST_F32: return launch_walls_st<ST_F32>(a, what, thermal, s);
+    case ST_F16: return launch_walls_st<ST_F16>(a, what, thermal, s);
+    default: return launch_walls_st<ST_BF16>(a, what, thermal, s);
   }
 }
 

@@ -183,7 +183,8 @@ hlbm_status hlbm_load(hlbm_ctx* ctx, const void* host_buf, size_t bytes);
 long long hlbm_step_count(const hlbm_ctx* ctx);
 
 /* Schedule of the fused periodic step (wall-bounded contexts accept and
- * ignore it: they have one schedule): tile rows per CTA (2D: 4, 8 or 16; D3Q39: 4
+ * ignore it: they have one schedule).  A context without one (none set, or
+ * 0, 0, 0) picks its kernel by size, kind and alignment.  Otherwise: tile rows per CTA (2D: 4, 8 or 16; D3Q39: 4
  * or 8; 0 = default 8), nodes per thread (1, or 2 on paired FP32 lanes
  * with 8 or 16 rows; 0 = default 2; D2Q37 only) and persistent CTAs that
  * prefetch their next tile (0 = default off, 1 = off, 2 = on, 3 = on and, on

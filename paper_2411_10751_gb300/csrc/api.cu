@@ -30,6 +30,7 @@ struct hlbm_ctx {
   int rows = 8;
   int npt = 2;
   int persistent = 0;
+  bool auto_schedule = true;      // no schedule set: the step picks its kernel by size
   bool multistep = false;         // D2Q37: one persistent launch for many steps (tile-row counters)
   unsigned gen = 0;               // multi-step kernel: steps run since the counters were zeroed
 
@@ -351,6 +352,12 @@ const CUtensorMap* tensor_map_at(hlbm_ctx* c, const void* base, int wb, int hb, 
 
 const CUtensorMap* tensor_map(hlbm_ctx* c, int buf, int wb, int hb) { return tensor_map_at(c, c->pop[buf], wb, hb); }
 
+// Whether the D2Q37 step runs without staging (direct.cu): contexts without a
+// schedule of their own; the hook that drops TMA copies needs the staged path.
+bool use_direct(const hlbm_ctx* c) {
+  return c->auto_schedule && !c->debug_skip_tma && direct_d2q37(c->kind, c->nx, c->ny, c->tma_ok);
+}
+
 cudaError_t launch_step(hlbm_ctx* c, StepArgs a, bool moments) {
   if (c->lattice != 0) {
     // persistent whole-row kernel: box of 256 / nx rows, and single rows
@@ -377,6 +384,7 @@ cudaError_t launch_step(hlbm_ctx* c, StepArgs a, bool moments) {
     }
     return launch_step_d3q39(a, c->kind, c->storage, moments, c->rows, c->npt, tm, c->stream);
   }
+  if (!moments && use_direct(c)) return launch_direct_d2q37(a, c->kind, c->storage, c->stream);
   CUtensorMap maps[2];
   std::memset(maps, 0, sizeof(maps));
   a.tma_store = 0;
@@ -954,12 +962,14 @@ hlbm_status hlbm_set_tile(hlbm_ctx* c, int rows, int nodes_per_thread, int persi
   if (!c) return HLBM_EINVAL;
   if (persistent < 0 || persistent > 3)
     return fail(c, HLBM_EINVAL, "persistent must be 0 (default off), 1 (off), 2 (on) or 3 (multi-step)");
+  const bool automatic = rows == 0 && nodes_per_thread == 0 && persistent == 0;
   if (rows == 0) rows = 8;
   if (nodes_per_thread == 0) nodes_per_thread = 2;
   if (rows != 4 && rows != 8 && rows != 16) return fail(c, HLBM_EINVAL, "rows must be 4, 8 or 16");
   if (nodes_per_thread != 1 && nodes_per_thread != 2) return fail(c, HLBM_EINVAL, "nodes_per_thread must be 1 or 2");
   if (nodes_per_thread == 2 && rows == 4) return fail(c, HLBM_EINVAL, "two nodes per thread need 8 or 16 rows");
   if (c->lattice == 1 && rows == 16) return fail(c, HLBM_EINVAL, "D3Q39 tiles have 4 or 8 rows");
+  c->auto_schedule = automatic;
   c->rows = rows;
   c->npt = nodes_per_thread;
   c->persistent = (persistent >= 2) ? 1 : 0;

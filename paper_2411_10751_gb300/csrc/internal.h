@@ -39,6 +39,26 @@ int per_device_cached(std::atomic<int> (&cache)[kMaxDevicesCached], F&& compute)
   return n;
 }
 
+// Launches a kernel that may start while the launch before it on the stream
+// still runs (programmatic dependent launch, also inside a captured graph):
+// its blocks take free slots and run up to grid_dependency_wait()
+// (step_common.cuh) meanwhile.  The kernel must execute that wait before its
+// first access to memory that an earlier launch reads or writes.
+template <class... P>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const P&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 enum Kind : int {
   KIND_LOCAL = 0,    // sources need only the node itself (F_i)
   KIND_THERMAL = 1,  // + H_i: theta of the 2D / 3D nearest neighbours
@@ -137,6 +157,11 @@ struct InitArgs {
 // npt: nodes per thread (1, or 2 on float2 lanes; 8- and 16-row tiles).
 cudaError_t launch_step_d2q37(const StepArgs& a, int kind, int storage, bool moments, int rows, int npt,
                               const CUtensorMap* tmap, cudaStream_t s);
+// The D2Q37 step without staging (direct.cu): 32 x 8 tiles, populations pulled
+// straight into registers; and whether it is the faster one for a domain (tma:
+// the staged kernel could use TMA).
+bool direct_d2q37(int kind, int nx, int ny, bool tma);
+cudaError_t launch_direct_d2q37(const StepArgs& a, int kind, int storage, cudaStream_t s);
 // tmap: {whole-row box, single-row} maps of the input buffer for the persistent
 // whole-row kernel (nx = 32, 64, 128, 256), or null.
 cudaError_t launch_step_d3q39(const StepArgs& a, int kind, int storage, bool moments, int rows, int npt,

@@ -1,0 +1,176 @@
+// Fused pull-collide-source step on D2Q37 without staging: every thread pulls
+// its node's populations straight into registers.
+//
+// A block owns the same 32 x 8 tile as the staged kernel (step2d.cuh) with one
+// node per thread, and further warps take the nodes of the frame around it (the
+// 80 ring nodes of theta for H_i, or the 276 frame nodes of psi for F^SC) at
+// the same time: all of a tile's loads are in flight at once, whatever the row
+// pitch or the periodic edge, where the staged kernel needs 16-byte aligned
+// rows for its TMA boxes and otherwise fills its planes in two to five passes
+// per thread.  The frame's lines are the neighbour tiles' (L1 or L2).
+// Node arithmetic, tile and frame are those of the staged kernel, so the
+// results are the same bit for bit.
+#pragma once
+
+#include "step2d.cuh"
+
+namespace hlbm {
+
+template <int KIND>
+struct Direct2 {
+  static constexpr int BX = 32, BY = 8, OWN = BX * BY;
+  static constexpr int H = KIND == KIND_SC ? 3 : (KIND == KIND_THERMAL ? 1 : 0);
+  using Fr = Frame2<BX, BY, (H > 0 ? H : 1)>;
+  static constexpr int FRAME = H > 0 ? Fr::count : 0;
+  static constexpr int NT = OWN + (FRAME + 31) / 32 * 32;
+};
+
+// v mod n for v >= -n
+__device__ __forceinline__ int wrap_up(int v, int n) {
+  if (v < 0) return v + n;
+  if (v >= n) v -= n;
+  return v < n ? v : v % n;
+}
+
+template <int ST, int KIND>
+__device__ __forceinline__ void direct_tile(const StepArgs& a, float* aux, int x0, int y0) {
+  using C = Codec<ST>;
+  using T = typename C::T;
+  using L = D2Q37;
+  using D = Direct2<KIND>;
+  using Fr = typename D::Fr;
+  constexpr int BX = D::BX, H = D::H;
+  constexpr float Dc = (float)(2.0 * L::cs2);
+  constexpr float inv_c0 = (float)(1.0 / L::c0);
+  const int nx = a.nx, ny = a.ny, tid = threadIdx.x;
+  const bool own = tid < D::OWN;
+  // region coordinates of this thread's node
+  int i = (tid & (BX - 1)) + H, j = tid / BX + H;
+  if constexpr (H > 0)
+    if (!own) Fr::pos(min(tid - D::OWN, D::FRAME - 1), i, j);
+  const int xr = x0 - H + i, yr = y0 - H + j;
+  const int x = wrap_up(xr, nx), y = wrap_up(yr, ny), node = y * nx + x;
+  const bool active = own && xr < nx && yr < ny;
+  float g[37];
+  gather<L, C>(static_cast<const T*>(a.fin), a.N, nx, ny, 1, x, y, 0, g);
+  if constexpr (H > 0) {
+    if (!own) {
+      if (tid - D::OWN < D::FRAME) {
+        float f;
+        if constexpr (KIND == KIND_SC) {
+          float hl;
+          const float hd = density_h<L>(g, hl);
+          f = psi_of<L>(a, hd, hl);
+        } else {
+          f = theta_bar_local<L>(a, g, node, y);
+        }
+        aux[frm<Fr>(j * Fr::SW + i)] = f;
+      }
+      __syncthreads();
+      return;
+    }
+  }
+  float dr, dr_l, acc, J[3], Pih;
+  moments_h<L>(g, dr, dr_l, acc, J, Pih);
+  const float rho = vadd(a.rho0, dr);
+  float ga[3];
+  accel<2>(a, node, y, ga);
+  float Fx = vmul(rho, ga[0]), Fy = vmul(rho, ga[1]), sigma = 0.f;
+  const float* ap = aux + j * Fr::SW + i;
+  if constexpr (KIND == KIND_SC) {
+    const float psi = psi_of<L>(a, dr, dr_l);
+    aux[frm<Fr>(j * Fr::SW + i)] = psi;
+    __syncthreads();
+    // F^SC = -G psi(x) sum_i w_i psi(x + c_i) c_i with G = -1
+    float sx = 0.f, sy = 0.f;
+    static_for<L::NPAIR>([&](auto P) {
+      constexpr int q = 2 * P + 1;
+      constexpr int cx = L::c(q, 0), cy = L::c(q, 1);
+      const float dpsi = ap[cy * Fr::SW + cx] - ap[-cy * Fr::SW - cx];
+      if constexpr (cx != 0) sx = vfma((float)(L::w(q) * cx), dpsi, sx);
+      if constexpr (cy != 0) sy = vfma((float)(L::w(q) * cy), dpsi, sy);
+    });
+    const float fsx = vmul(psi, sx), fsy = vmul(psi, sy);
+    Fx = vadd(Fx, fsx);
+    Fy = vadd(Fy, fsy);
+    // P_i trace coefficient (Eq. 3.12): sigma = p_coef |F^SC|^2 / psi^2
+    sigma = (psi > 0.f) ? a.p_coef * (fsx * fsx + fsy * fsy) * rcp_nr(psi * psi) : 0.f;
+  }
+  const float inv_rho = rcp_nr(rho);
+  const float ux = vmul(vfma(0.5f, Fx, J[0]), inv_rho), uy = vmul(vfma(0.5f, Fy, J[1]), inv_rho);
+  const float uu = vfma(ux, ux, vmul(uy, uy));
+  const float G2 = vfma(Dc, sigma, vmul(2.f, vfma(ux, Fx, vmul(uy, Fy))));
+  const float tb = vmul(vmul(vfma(0.5f, G2, vsub(Pih, vmul(rho, uu))), inv_rho), 1.f / Dc);
+  NodeSrcT<float> s;
+  s.hG[0] = s.hG[1] = s.hG[2] = 0.f;
+  if constexpr (KIND == KIND_THERMAL) {
+    aux[frm<Fr>(j * Fr::SW + i)] = tb;
+    __syncthreads();
+    const float gtx = 0.5f * (ap[1] - ap[-1]), gty = 0.5f * (ap[Fr::SW] - ap[-Fr::SW]);
+    // s^(3) += rho theta (1 - 1/Pr) [delta grad_xi theta], grad_xi = c0 grad
+    const float hc = vmul(vmul(rho, vadd(1.f, tb)), a.h_coef * (float)L::c0);
+    s.hG[0] = vmul(hc, gtx);
+    s.hG[1] = vmul(hc, gty);
+  }
+  if (!active) return;
+  s.dr = 0.f;  // density deviation re-enters in apply_poly_h
+  s.rho = rho;
+  s.tb = a.isothermal ? 0.f : tb;
+  s.u[0] = vmul(ux, inv_c0);
+  s.u[1] = vmul(uy, inv_c0);
+  s.u[2] = 0.f;
+  s.F[0] = vmul(Fx, inv_c0);
+  s.F[1] = vmul(Fy, inv_c0);
+  s.F[2] = 0.f;
+  s.sigma = sigma;
+  float K[15];
+  poly2<L>(s, a.omega, a.beta, K);
+  const float om1 = 1.f - a.omega;
+  K[0] = vfma(-om1, acc, K[0]);
+  if constexpr (KIND == KIND_SC) K[0] = vadd(K[0], dr_l);
+  apply_poly_h<L, 15>(g, K, om1, dr);
+  const uint32_t salt = std::is_same<T, float>::value ? 0u : node_salt(node, g[0]);
+  if (!HLBM_IN(node, a.N, DBG_STORE)) return;
+  T* __restrict__ fout = static_cast<T*>(a.fout) + node;
+  static_for<37>([&](auto I) {
+    constexpr int q = I;
+    fout[(size_t)q * (size_t)a.N] = round_store<T>(g[q], pop_bits(salt, q));
+  });
+}
+
+// PER: blocks per SM that the registers are sized for
+template <int ST, int KIND, int PER>
+__global__ void __launch_bounds__(Direct2<KIND>::NT, PER) step2d_direct_kernel(const __grid_constant__ StepArgs a) {
+  using D = Direct2<KIND>;
+  __shared__ float aux[D::H > 0 ? D::Fr::SW * D::Fr::SH : 1];
+  grid_dependency_wait();
+  direct_tile<ST, KIND>(a, aux, blockIdx.x * D::BX, blockIdx.y * D::BY);
+}
+
+// Blocks per SM of the throughput form: 80 registers leave 2 thermal and 3
+// body-force blocks (3 and 4, with 56 and 64 registers, spill and gain nothing:
+// 901 x 899 58.2 against 58.5 us, 47.3 against 48.3 us); the pseudopotential
+// block of 17 warps at 56 registers with 100 B of spills pays off as soon as
+// the tiles outnumber the SMs (641 x 639 FP32 52.0 -> 45.9 us; on fewer tiles
+// one block per SM without spills: 64 x 64 5.0 -> 4.4 us).
+template <int KIND>
+constexpr int direct2_per_sm() {
+  return KIND == KIND_LOCAL ? 3 : 2;
+}
+
+template <int ST, int KIND, int PER>
+cudaError_t launch_direct2(const StepArgs& a, dim3 grid, cudaStream_t s) {
+  return launch_pdl(step2d_direct_kernel<ST, KIND, PER>, grid, Direct2<KIND>::NT, 0, s, a);
+}
+
+template <int ST>
+cudaError_t launch_direct2_st(const StepArgs& a, int kind, int sms, cudaStream_t s) {
+  const dim3 grid((a.nx + 31) / 32, (a.ny + 7) / 8);
+  if (kind == KIND_SC)
+    return (int)(grid.x * grid.y) <= sms ? launch_direct2<ST, KIND_SC, 1>(a, grid, s)
+                                         : launch_direct2<ST, KIND_SC, direct2_per_sm<KIND_SC>()>(a, grid, s);
+  if (kind == KIND_THERMAL) return launch_direct2<ST, KIND_THERMAL, direct2_per_sm<KIND_THERMAL>()>(a, grid, s);
+  return launch_direct2<ST, KIND_LOCAL, direct2_per_sm<KIND_LOCAL>()>(a, grid, s);
+}
+
+}  // namespace hlbm

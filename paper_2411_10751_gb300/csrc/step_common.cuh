@@ -88,6 +88,11 @@ __device__ __forceinline__ bool dbg_ok(long long i, long long n, int site) {
 #define HLBM_IN(i, n, site) true
 #endif
 
+// --------------------------------------------------- dependent launches
+// Waits until the launch before this one on the stream has completed and its
+// writes are visible (launch_pdl; otherwise it returns at once).
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------ codecs
 template <int S> struct Codec;
 template <> struct Codec<ST_F32> {

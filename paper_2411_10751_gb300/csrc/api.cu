@@ -267,6 +267,23 @@ void drop_graphs(hlbm_ctx* c) {
     }
 }
 
+// Whether a context without a schedule runs the persistent kernels (D2Q37
+// staged tiles, D3Q39 whole rows).  Their CTAs take ordered tiles and hold the
+// next one in flight, which pays once a step streams from HBM, i.e. when the two
+// buffers outgrow what L2 (129 MB) keeps of them; inside it the hardware's own
+// block scheduling is faster.  us per step, one CTA per tile against
+// persistent, FP32 unless stated: thermal 512 x 512 (78 MB) 16.7 / 18.0, 576 x 576
+// (98 MB) 21.4 / 19.6, 1024 x 1024 60.9 / 54.9; pseudopotential 576 x 576 35.9 /
+// 34.8, 1024 x 1024 95.5 / 89.4; D3Q39 64^3 (82 MB) 14.3 / 15.0, 128^3 136.2 / 98.8,
+// 128^3 FP16 97.1 / 79.9.  Not for D2Q37 in 16 bits, whose persistent form has 3
+// CTAs per SM instead of 4 (thermal 1024 x 1024 45.4 / 48.8), nor for the body
+// force alone, which gains at some sizes (1024 x 1024 54.1 / 53.1) and loses at
+// others (1536 x 1536 109.1 / 112.4).
+int auto_persistent(const hlbm_ctx* c) {
+  if (2.0 * c->Q * (double)c->N * (double)c->elem < 96e6) return 0;
+  return c->lattice == HLBM_D3Q39 || (c->storage == ST_F32 && c->kind != KIND_LOCAL) ? 1 : 0;
+}
+
 StepArgs make_args(const hlbm_ctx* c) {
   StepArgs a{};
   a.N = c->N;
@@ -288,7 +305,7 @@ StepArgs make_args(const hlbm_ctx* c) {
   split_ff(c->p.eos == 0 ? c->p.eos_b : 0.25 * c->p.eos_b, a.psi_kb);
   a.status = c->status;
   a.tma = c->tma_ok ? 1 : 0;
-  a.persistent = c->persistent;
+  a.persistent = c->auto_schedule ? auto_persistent(c) : c->persistent;
   a.tile_ctr = c->tile_ctr;
   a.wait_ns = c->wait_ns;
   a.debug_skip_tma = c->debug_skip_tma;

@@ -239,10 +239,9 @@ hlbm_status hlbm_adjoint_run(hlbm_ctx* ctx, int steps, int ckpt_every, void* wor
  * sizes, sources and parameters, one storage type -- together, with ONE
  * persistent kernel launch per time step (replayed from a CUDA graph of two
  * steps): resident CTAs take (domain, tile) items of every domain from a work
- * list through a device counter and run the single-domain tile code (32 x 8
- * tiles, two nodes per thread; 32 x 4 tiles, one node per thread, for the
- * pseudopotential kind), so each context's state equals that of hlbm_step
- * with those schedules bit for bit.  The contexts must be initialised;
+ * list through a device counter and run the single-domain step without staging
+ * on 32 x 8 tiles, so each context's state equals that of hlbm_step on 8-row
+ * tiles bit for bit.  The contexts must be initialised;
  * hlbm_batch_create moves them onto the batch's stream, so their own calls
  * stay ordered with batch steps.  Each context's state and step count advance
  * as if hlbm_step had been called; hlbm_moments / hlbm_diag / hlbm_save work

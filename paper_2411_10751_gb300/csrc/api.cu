@@ -367,8 +367,6 @@ const CUtensorMap* tensor_map_at(hlbm_ctx* c, const void* base, int wb, int hb, 
   return &c->tmaps.back().map;
 }
 
-const CUtensorMap* tensor_map(hlbm_ctx* c, int buf, int wb, int hb) { return tensor_map_at(c, c->pop[buf], wb, hb); }
-
 // Whether the D2Q37 step runs without staging (direct.cu): contexts without a
 // schedule of their own; the hook that drops TMA copies needs the staged path.
 bool use_direct(const hlbm_ctx* c) {
@@ -604,7 +602,6 @@ StepArgs ctx_step_args(hlbm_ctx* c, int parity) {
   a.persistent = 0;
   return a;
 }
-const CUtensorMap* ctx_tensor_map(hlbm_ctx* c, int buf, int wb, int hb) { return tensor_map(c, buf, wb, hb); }
 int ctx_cur(const hlbm_ctx* c) { return c->cur; }
 void ctx_advance(hlbm_ctx* c, int steps) {
   c->cur ^= (steps & 1);

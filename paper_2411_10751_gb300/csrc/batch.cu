@@ -1,90 +1,44 @@
 // Batched step: many independent periodic D2Q37 domains (any sizes, sources
 // and parameters) advanced by ONE persistent launch per time step, replayed
-// from a CUDA graph.  Resident CTAs (all of the same shape: 128 threads,
-// shared memory for the largest tile) take (domain, tile) items from a global
-// work list in order through a device counter, dispatch on the domain's
-// source kind and run exactly the single-domain kernel's tile code
-// (process_tile): 32 x 8 tiles with two nodes per thread for the body-force
-// and thermal kinds, 32 x 4 tiles with one node per thread for the
-// pseudopotential kind (its frame of psi values is three nodes wide; a 4-row
-// tile keeps its staging at 67 KB FP32, so three CTAs fit on an SM whatever
-// kind they run).  The pseudopotential tiles, the slowest, come first in the
-// work list, so the launch ends on short tiles.  Each domain's step arguments
-// (for both buffer parities) and its TMA tensor maps are read from device
-// memory.
+// from a CUDA graph.  Resident CTAs (all of the same shape: 352 threads) take
+// (domain, tile) items from a global work list in order through a device
+// counter and run the step without staging (direct_tile, step2d_direct.cuh) of
+// the domain's source kind on it: most tiles of small domains touch the
+// periodic edge or belong to rows that TMA cannot take, so staging them was a
+// synchronous gather into shared memory, and a block held 93 KB of it.  A tile's
+// 256 nodes take one thread each; the theta ring of the thermal kind runs
+// beside them on the last three warps, the 276 psi nodes of the pseudopotential
+// kind before them on all.  The pseudopotential tiles, the slowest, come first
+// in the work list, so the launch ends on short tiles.  Item and step arguments
+// are read from device memory one item ahead, by the last warps while the
+// others collide.  It is bound by instruction issue (53% of the slots) and the
+// loads' latency at 22 warps per SM: 256 domains, 6.4 M nodes, FP32, 770 -> 564 us
+// a step (the staged form spent 62 warp instructions per node, this one 45).
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <string>
 #include <vector>
 
-#include <cudaTypedefs.h>
-
 #include "hlbm.h"
 #include "internal.h"
-#include "step2d.cuh"
+#include "step2d_direct.cuh"
 
 namespace hlbm {
 namespace {
 
-// tile rows and nodes per thread of a kind (256 threads for every kind)
-template <int KIND>
-constexpr int kind_rows() {
-  return 8;
-}
-template <int KIND>
-constexpr int kind_npt() {
-  return 1;
-}
-constexpr int kThreads = 256;
-int kind_rows_rt(int) { return 8; }
+constexpr int kThreads = Direct2<KIND_THERMAL>::NT;
+constexpr int kOwn = Direct2<KIND_THERMAL>::OWN;
+constexpr int kAux = Direct2<KIND_SC>::Fr::SW * Direct2<KIND_SC>::Fr::SH;
 
-template <int ST>
-constexpr int batch_smem() {
-  constexpr int a = Cfg2<ST, KIND_LOCAL, false, 8>::SMEM, b = Cfg2<ST, KIND_THERMAL, false, 8>::SMEM,
-                c = Cfg2<ST, KIND_SC, false, 8>::SMEM;
-  return a > b ? (a > c ? a : c) : (b > c ? b : c);
-}
-
-struct alignas(64) BatchDomain {
-  CUtensorMap tmap[2];    // input maps of buffer 0 / 1 (box of the domain's kind)
-  StepArgs args[2];       // args[p]: reads buffer p, writes buffer p ^ 1
-  int kind;
-  int tiles_x;
-  int cur;                // buffer holding the state at the start of the batch call
-  int has_map;
+struct BatchDomain {
+  StepArgs args[2];       // args[0]: from the buffer that holds the state at the start of the batch call, args[1]: back
 };
-
-template <int ST, int KIND>
-__device__ __forceinline__ bool batch_tile(const BatchDomain& dom, const StepArgs& a, unsigned char* smem, int x0,
-                                           int y0, int par, uint32_t& phase) {
-  constexpr int BY = kind_rows<KIND>();
-  using Cf = Cfg2<ST, KIND, false, BY>;
-  typename Cf::T* sp = reinterpret_cast<typename Cf::T*>(smem);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + batch_smem<ST>() - 128);
-  const int tid = threadIdx.y * 32 + threadIdx.x;
-  if (dom.has_map && tile_boxed<Cf>(a, x0, y0) && ((smem_u32(smem) & 127u) == 0)) {
-    if (tid == 0) {
-      fence_proxy_async_smem();   // the previous tile's generic accesses of the buffer come first
-      issue_tile<Cf>(sp, &dom.tmap[par], bar, x0, y0, a.debug_skip_tma, a.nx, a.ny);
-    }
-    const bool ok = mbar_wait_bounded(bar, phase, a.wait_ns);
-    phase ^= 1u;
-    if (!__syncthreads_and(ok)) {
-      // copies did not complete: report, give in-flight copies a second
-      // bounded wait, and stop this CTA (the batch is then in an error state)
-      if (tid == 0) atomicExch(a.status, (int)5 /* HLBM_ETIMEOUT */);
-      mbar_wait_bounded(bar, phase ^ 1u, a.wait_ns);
-      __syncthreads();
-      return false;
-    }
-  } else {
-    fill_tile_wrapped<Cf, kThreads>(a, a.fin, sp, x0, y0, tid);
-    __syncthreads();
-  }
-  process_tile<ST, KIND, false, BY, kind_npt<KIND>(), false>(a, nullptr, smem, x0, y0, a.fout, [] {});
-  return true;
-}
+struct BatchItem {
+  int domain, kind, x0, y0;
+};
+constexpr int kArgWords = (int)(sizeof(StepArgs) / 4);
+static_assert(sizeof(StepArgs) % 8 == 0 && sizeof(BatchItem) == 16, "copied by words");
 
 // One step of every domain: CTAs take work-list items (T = nitems) through
 // the counter; a launch of G CTAs takes exactly T + G values (each CTA ends
@@ -92,44 +46,46 @@ __device__ __forceinline__ bool batch_tile(const BatchDomain& dom, const StepArg
 // the value modulo T + G.
 template <int ST>
 __global__ void __launch_bounds__(kThreads, 2)
-    batch_step_kernel(const BatchDomain* __restrict__ doms, const int2* __restrict__ items, int nitems, int flip,
+    batch_step_kernel(const BatchDomain* __restrict__ doms, const BatchItem* __restrict__ items, int nitems, int flip,
                       unsigned long long* ctr) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ int s_item;
-  const int tid = threadIdx.y * 32 + threadIdx.x;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + batch_smem<ST>() - 128);
-  // thread 0 takes the counter one item ahead and keeps the raw value until
-  // the next item starts, so the atomic's round trip overlaps a whole tile
-  unsigned long long nxt_raw = 0;
+  __shared__ float aux[kAux];
+  __shared__ __align__(16) unsigned s_args[2][kArgWords];
+  __shared__ BatchItem s_item[2];
+  __shared__ int s_next[4];                            // item index of turn n at n mod 4
+  const int tid = threadIdx.x;
+  // thread 0 takes item indices two turns ahead and keeps the last as the
+  // counter's raw value, so the atomic's round trip overlaps a whole tile
+  unsigned long long raw = 0;
   const unsigned long long period = (unsigned long long)nitems + gridDim.x;
+  const auto fetch = [&](int turn, int first, int n) {   // threads first .. first + n - 1: item and arguments of a turn
+    const int gi = s_next[turn & 3];
+    if (gi >= nitems) return;
+    const BatchItem it = items[gi];
+    const unsigned* src = reinterpret_cast<const unsigned*>(&doms[it.domain].args[flip]);
+    for (int w = tid - first; w < kArgWords; w += n) s_args[turn & 1][w] = __ldg(src + w);
+    if (tid == first) s_item[turn & 1] = it;
+  };
   if (tid == 0) {
-    mbar_init(bar, 1);
-    fence_mbar_init();
-    nxt_raw = atomicAdd(ctr, 1ull);
+    const int g0 = (int)(atomicAdd(ctr, 1ull) % period);
+    s_next[0] = g0;
+    if (g0 < nitems) raw = atomicAdd(ctr, 1ull);
   }
-  uint32_t phase = 0;
-  for (;;) {
-    if (tid == 0) {
-      const int gi = (int)(nxt_raw % period);
-      s_item = gi;
-      if (gi < nitems) nxt_raw = atomicAdd(ctr, 1ull);
+  __syncthreads();
+  fetch(0, 0, kThreads);
+  for (int turn = 0;; ++turn) {
+    if (tid == 0 && s_next[turn & 3] < nitems) {
+      const int gi = (int)(raw % period);
+      s_next[(turn + 1) & 3] = gi;   // (a slow warp may still read the slot of turn - 1)
+      if (gi < nitems) raw = atomicAdd(ctr, 1ull);
     }
-    __syncthreads();
-    const int gi = s_item;
-    if (gi >= nitems) break;
-    const int2 it = items[gi];                   // (domain, tile)
-    const BatchDomain& dom = doms[it.x];
-    const int par = dom.cur ^ flip;
-    const StepArgs& a = dom.args[par];
-    const int t = it.y;
-    const int ty = t / dom.tiles_x;
-    const int x0 = (t - ty * dom.tiles_x) * 32;
-    bool ok;
-    if (dom.kind == KIND_SC) ok = batch_tile<ST, KIND_SC>(dom, a, smem, x0, ty * kind_rows<KIND_SC>(), par, phase);
-    else if (dom.kind == KIND_THERMAL) ok = batch_tile<ST, KIND_THERMAL>(dom, a, smem, x0, ty * 8, par, phase);
-    else ok = batch_tile<ST, KIND_LOCAL>(dom, a, smem, x0, ty * 8, par, phase);
-    if (!ok) return;
-    __syncthreads();   // the staging buffer and s_item are reused
+    __syncthreads();   // this turn's item and the next one's index are there; aux is free
+    if (s_next[turn & 3] >= nitems) return;
+    const StepArgs& a = *reinterpret_cast<const StepArgs*>(s_args[turn & 1]);
+    const BatchItem it = s_item[turn & 1];
+    if (it.kind == KIND_SC) direct_tile<ST, KIND_SC, kThreads>(a, aux, it.x0, it.y0);
+    else if (it.kind == KIND_THERMAL) direct_tile<ST, KIND_THERMAL, kThreads>(a, aux, it.x0, it.y0);
+    else direct_tile<ST, KIND_LOCAL, kThreads>(a, aux, it.x0, it.y0);
+    if (tid >= kOwn) fetch(turn + 1, kOwn, kThreads - kOwn);
   }
 }
 
@@ -138,29 +94,17 @@ int batch_grid(int nitems) {
   int per_sm = 0, sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_step_kernel<ST>, kThreads, batch_smem<ST>());
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_step_kernel<ST>, kThreads, 0);
   if (per_sm < 1) per_sm = 1;
   return std::max(1, std::min(nitems, sms * per_sm));
 }
 
 template <int ST>
-cudaError_t launch_batch(const BatchDomain* doms, const int2* items, int nitems, int grid, int flip,
+cudaError_t launch_batch(const BatchDomain* doms, const BatchItem* items, int nitems, int grid, int flip,
                          unsigned long long* ctr, cudaStream_t s) {
   if (nitems <= 0) return cudaSuccess;
-  batch_step_kernel<ST><<<grid, dim3(32, kThreads / 32, 1), batch_smem<ST>(), s>>>(doms, items, nitems, flip, ctr);
+  batch_step_kernel<ST><<<grid, kThreads, 0, s>>>(doms, items, nitems, flip, ctr);
   return cudaGetLastError();
-}
-
-template <int ST>
-cudaError_t configure_batch() {
-  return cudaFuncSetAttribute(batch_step_kernel<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, batch_smem<ST>());
-}
-
-template <int ST>
-void box_for_kind(int kind, int& wb, int& hb) {
-  if (kind == KIND_SC) box_of<ST, KIND_SC, false, 8>(wb, hb);
-  else if (kind == KIND_THERMAL) box_of<ST, KIND_THERMAL, false, 8>(wb, hb);
-  else box_of<ST, KIND_LOCAL, false, 8>(wb, hb);
 }
 
 }  // namespace
@@ -168,17 +112,17 @@ void box_for_kind(int kind, int& wb, int& hb) {
 // Host-side helpers the C ABI (api.cu) uses; the batch owns the device arrays.
 struct BatchDevice {
   BatchDomain* doms = nullptr;
-  int2* items = nullptr;
+  BatchItem* items = nullptr;
   unsigned long long* ctr = nullptr;   // the persistent launch's item counter (zeroed once)
   int nitems = 0;
 };
 
-cudaError_t batch_upload(const std::vector<BatchDomain>& host, const std::vector<int2>& items, BatchDevice& dev,
+cudaError_t batch_upload(const std::vector<BatchDomain>& host, const std::vector<BatchItem>& items, BatchDevice& dev,
                          cudaStream_t s) {
   if (!dev.doms) {
     cudaError_t e = cudaMalloc(&dev.doms, host.size() * sizeof(BatchDomain));
     if (e != cudaSuccess) return e;
-    e = cudaMalloc(&dev.items, items.size() * sizeof(int2));
+    e = cudaMalloc(&dev.items, items.size() * sizeof(BatchItem));
     if (e != cudaSuccess) return e;
     e = cudaMalloc(&dev.ctr, sizeof(unsigned long long));
     if (e != cudaSuccess) return e;
@@ -187,7 +131,7 @@ cudaError_t batch_upload(const std::vector<BatchDomain>& host, const std::vector
   }
   cudaError_t e = cudaMemcpyAsync(dev.doms, host.data(), host.size() * sizeof(BatchDomain), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(dev.items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
+    e = cudaMemcpyAsync(dev.items, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, s);
   dev.nitems = (int)items.size();
   return e;
 }
@@ -202,7 +146,7 @@ struct hlbm_batch {
   int storage = 0;
   cudaStream_t stream = nullptr;
   std::vector<BatchDomain> host;
-  std::vector<int2> items;        // (domain, tile), the pseudopotential kind's tiles first
+  std::vector<BatchItem> items;   // the pseudopotential kind's tiles first
   int grid = 0;                   // resident CTAs of the persistent launch
   BatchDevice dev;
   cudaGraphExec_t graph = nullptr;
@@ -213,7 +157,6 @@ struct hlbm_batch {
 namespace hlbm {
 bool ctx_batchable(const hlbm_ctx* c, int* storage, int* kind, int* nx, int* ny);
 StepArgs ctx_step_args(hlbm_ctx* c, int parity);
-const CUtensorMap* ctx_tensor_map(hlbm_ctx* c, int buf, int wb, int hb);
 int ctx_cur(const hlbm_ctx* c);
 void ctx_advance(hlbm_ctx* c, int steps);
 }  // namespace hlbm
@@ -248,13 +191,6 @@ hlbm_status hlbm_batch_create(int n, hlbm_ctx* const* ctxs, hlbm_batch** out) {
     hlbm_synchronize(c);
     hlbm_set_stream(c, b->stream);
   }
-  cudaError_t e = storage == ST_F32 ? configure_batch<ST_F32>()
-                  : storage == ST_F16 ? configure_batch<ST_F16>()
-                                      : configure_batch<ST_BF16>();
-  if (e != cudaSuccess) {
-    hlbm_batch_destroy(b);
-    return HLBM_ECUDA;
-  }
   *out = b;
   return HLBM_OK;
 }
@@ -262,7 +198,7 @@ hlbm_status hlbm_batch_create(int n, hlbm_ctx* const* ctxs, hlbm_batch** out) {
 static hlbm_status batch_refresh(hlbm_batch* b) {
   b->host.assign(b->ctxs.size(), BatchDomain{});
   b->items.clear();
-  std::vector<int2> heavy, light;   // pseudopotential tiles (compute-bound) and the others (HBM-bound)
+  std::vector<BatchItem> heavy, light;   // pseudopotential tiles (compute-bound) and the others (HBM-bound)
   for (int kind : {(int)KIND_SC, (int)KIND_THERMAL, (int)KIND_LOCAL}) {
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
       hlbm_ctx* c = b->ctxs[k];
@@ -271,25 +207,11 @@ static hlbm_status batch_refresh(hlbm_batch* b) {
       if (dkind != kind) continue;
       BatchDomain& d = b->host[k];
       std::memset(&d, 0, sizeof(d));
-      d.kind = dkind;
-      d.tiles_x = (nx + 31) / 32;
-      d.cur = ctx_cur(c);
-      d.args[0] = ctx_step_args(c, 0);
-      d.args[1] = ctx_step_args(c, 1);
-      int wb = 0, hb = 0;
-      if (st == ST_F32) box_for_kind<ST_F32>(dkind, wb, hb);
-      else if (st == ST_F16) box_for_kind<ST_F16>(dkind, wb, hb);
-      else box_for_kind<ST_BF16>(dkind, wb, hb);
-      const CUtensorMap* m0 = d.args[0].tma ? ctx_tensor_map(c, 0, wb, hb) : nullptr;
-      const CUtensorMap* m1 = d.args[0].tma ? ctx_tensor_map(c, 1, wb, hb) : nullptr;
-      d.has_map = (m0 && m1) ? 1 : 0;
-      if (d.has_map) {
-        d.tmap[0] = *m0;
-        d.tmap[1] = *m1;
-      }
-      const int rows = kind_rows_rt(dkind);
-      const int tiles = d.tiles_x * ((ny + rows - 1) / rows);
-      for (int t = 0; t < tiles; ++t) (dkind == KIND_SC ? heavy : light).push_back(make_int2((int)k, t));
+      const int cur = ctx_cur(c);
+      d.args[0] = ctx_step_args(c, cur);
+      d.args[1] = ctx_step_args(c, cur ^ 1);
+      for (int y0 = 0; y0 < ny; y0 += 8)
+        for (int x0 = 0; x0 < nx; x0 += 32) (dkind == KIND_SC ? heavy : light).push_back(BatchItem{(int)k, dkind, x0, y0});
     }
   }
   // the slow tiles first, so the launch ends on short ones (measured against

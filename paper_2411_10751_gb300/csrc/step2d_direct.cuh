@@ -32,7 +32,24 @@ __device__ __forceinline__ int wrap_up(int v, int n) {
   return v < n ? v : v % n;
 }
 
-template <int ST, int KIND>
+// theta or psi of a frame node, from its pulled populations
+template <int KIND>
+__device__ __forceinline__ float frame_value(const StepArgs& a, float (&g)[37], int node, int y) {
+  using L = D2Q37;
+  if constexpr (KIND == KIND_SC) {
+    float hl;
+    const float hd = density_h<L>(g, hl);
+    return psi_of<L>(a, hd, hl);
+  } else {
+    return theta_bar_local<L>(a, g, node, y);
+  }
+}
+
+// The step of the tile at (x0, y0) by the block's NT threads; aux: the frame
+// array in shared memory (free once every thread has returned).  Where NT has no
+// room for the frame beside the tile (the batched step's pseudopotential tiles)
+// all threads take the frame's nodes first.
+template <int ST, int KIND, int NT>
 __device__ __forceinline__ void direct_tile(const StepArgs& a, float* aux, int x0, int y0) {
   using C = Codec<ST>;
   using T = typename C::T;
@@ -43,29 +60,35 @@ __device__ __forceinline__ void direct_tile(const StepArgs& a, float* aux, int x
   constexpr float Dc = (float)(2.0 * L::cs2);
   constexpr float inv_c0 = (float)(1.0 / L::c0);
   const int nx = a.nx, ny = a.ny, tid = threadIdx.x;
+  constexpr bool BESIDE = D::OWN + D::FRAME <= NT;
+  const T* fin = static_cast<const T*>(a.fin);
   const bool own = tid < D::OWN;
+  float g[37];
+  if constexpr (!BESIDE) {
+    for (int k = tid; k < D::FRAME; k += NT) {
+      int fi, fj;
+      Fr::pos(k, fi, fj);
+      const int fx = wrap_up(x0 - H + fi, nx), fy = wrap_up(y0 - H + fj, ny);
+      gather<L, C>(fin, a.N, nx, ny, 1, fx, fy, 0, g);
+      aux[frm<Fr>(fj * Fr::SW + fi)] = frame_value<KIND>(a, g, fy * nx + fx, fy);
+    }
+    if (!own) {
+      __syncthreads();
+      return;
+    }
+  }
   // region coordinates of this thread's node
   int i = (tid & (BX - 1)) + H, j = tid / BX + H;
-  if constexpr (H > 0)
+  if constexpr (H > 0 && BESIDE)
     if (!own) Fr::pos(min(tid - D::OWN, D::FRAME - 1), i, j);
   const int xr = x0 - H + i, yr = y0 - H + j;
   const int x = wrap_up(xr, nx), y = wrap_up(yr, ny), node = y * nx + x;
   const bool active = own && xr < nx && yr < ny;
-  float g[37];
-  gather<L, C>(static_cast<const T*>(a.fin), a.N, nx, ny, 1, x, y, 0, g);
-  if constexpr (H > 0) {
+  if (H == 0 && !own) return;
+  gather<L, C>(fin, a.N, nx, ny, 1, x, y, 0, g);
+  if constexpr (H > 0 && BESIDE) {
     if (!own) {
-      if (tid - D::OWN < D::FRAME) {
-        float f;
-        if constexpr (KIND == KIND_SC) {
-          float hl;
-          const float hd = density_h<L>(g, hl);
-          f = psi_of<L>(a, hd, hl);
-        } else {
-          f = theta_bar_local<L>(a, g, node, y);
-        }
-        aux[frm<Fr>(j * Fr::SW + i)] = f;
-      }
+      if (tid - D::OWN < D::FRAME) aux[frm<Fr>(j * Fr::SW + i)] = frame_value<KIND>(a, g, node, y);
       __syncthreads();
       return;
     }
@@ -144,7 +167,7 @@ __global__ void __launch_bounds__(Direct2<KIND>::NT, PER) step2d_direct_kernel(c
   using D = Direct2<KIND>;
   __shared__ float aux[D::H > 0 ? D::Fr::SW * D::Fr::SH : 1];
   grid_dependency_wait();
-  direct_tile<ST, KIND>(a, aux, blockIdx.x * D::BX, blockIdx.y * D::BY);
+  direct_tile<ST, KIND, D::NT>(a, aux, blockIdx.x * D::BX, blockIdx.y * D::BY);
 }
 
 // Blocks per SM of the throughput form: 80 registers leave 2 thermal and 3

@@ -124,7 +124,8 @@ typedef struct {
 typedef struct hlbm_ctx hlbm_ctx;
 
 /* Bytes of device memory a context needs (two population buffers, the force
- * field when HLBM_SRC_FORCE is set, diagnostics scratch).  0 on bad input. */
+ * field when HLBM_SRC_FORCE is set, a psi field with HLBM_SRC_SC, diagnostics
+ * scratch).  0 on bad input. */
 size_t hlbm_workspace_bytes(int lattice, int nx, int ny, int nz, const hlbm_source_params* p);
 
 /* Creates a context.  nx, ny (and nz for D3Q39) >= 7 so that the reach-3

@@ -125,9 +125,10 @@ Layout layout(int lattice, int nx, int ny, int nz, const hlbm_source_params* p) 
   // walls: two [4][N] FP32 moment fields (previous step, this step)
   L.mom_bytes = (p->flags & HLBM_WALLS) ? align256((size_t)4 * (size_t)N * 4) : 0;
   L.off_aux = L.off_mom + 2 * L.mom_bytes;
-  L.aux_bytes = (p->flags & HLBM_AA) ? align256((size_t)N * 4) : 0;
+  // in place: two neighbour fields; pseudopotential on two buffers: psi
+  L.aux_bytes = (p->flags & (HLBM_AA | HLBM_SRC_SC)) ? align256((size_t)N * 4) : 0;
   // walls: the completed unknowns of the six wall rows of each buffer, [6][37][nx] FP32
-  L.off_comp = L.off_aux + 2 * L.aux_bytes;
+  L.off_comp = L.off_aux + ((p->flags & HLBM_AA) ? 2 : 1) * L.aux_bytes;
   L.comp_bytes = (p->flags & HLBM_WALLS) ? align256((size_t)6 * 37 * (size_t)nx * 4) : 0;
   L.total = L.off_comp + 2 * L.comp_bytes;
   return L;
@@ -398,6 +399,13 @@ cudaError_t launch_step(hlbm_ctx* c, StepArgs a, bool moments) {
       }
     }
     return launch_step_d3q39(a, c->kind, c->storage, moments, c->rows, c->npt, tm, c->stream);
+  }
+  if (!moments && c->kind == KIND_SC && c->auto_schedule && !c->debug_skip_tma &&
+      two_launch_d2q37(c->storage, c->nx, c->ny, c->tma_ok)) {
+    a.aux_wr = c->aux[0];
+    a.aux_rd = c->aux[0];
+    const cudaError_t e = launch_psi_d2q37(a, c->storage, c->stream);
+    return e != cudaSuccess ? e : launch_direct_d2q37(a, KIND_SCF, c->storage, c->stream);
   }
   if (!moments && use_direct(c)) return launch_direct_d2q37(a, c->kind, c->storage, c->stream);
   CUtensorMap maps[2];

@@ -32,6 +32,27 @@ bool direct_d2q37(int kind, int nx, int ny, bool tma) {
   return tiles <= (long long)per * sm_count();
 }
 
+// Two launches read the populations twice but replace the frame's 1.08 pulls
+// and psi values per node by one psi value.  They pay off when the tiles exceed
+// one wave of blocks and the second read comes from L2 or the rows keep TMA out
+// (FP32 us per step, one launch / two: 320 x 320 15.1 / 11.5, 512 x 512 27.4 /
+// 23.8, 544 x 544 30.2 / 27.3, 640 x 640 37.8 / 39.2; 641 x 639 46.3 / 41.3, 901 x
+// 899 85.3 / 83.5, 1201 x 1199 146.3 / 139.1, FP16 133.9 / 124.4).  Aligned 16-bit
+// domains gain nothing (384 x 384 14.3 / 15.0, 512 x 512 23.1 / 23.5).
+bool two_launch_d2q37(int storage, int nx, int ny, bool tma) {
+  if (direct_d2q37(KIND_SC, nx, ny, true)) return false;   // one wave: a launch more costs more
+  return !tma || (storage == ST_F32 && 2.0 * 37 * 4 * (double)nx * ny < 96e6);
+}
+
+cudaError_t launch_psi_d2q37(const StepArgs& a, int storage, cudaStream_t s) {
+  const dim3 grid((a.nx + 31) / 32, (a.ny + 7) / 8);
+  switch (storage) {
+    case ST_F32: return launch_pdl(psi_kernel<ST_F32>, grid, dim3(256), 0, s, a);
+    case ST_F16: return launch_pdl(psi_kernel<ST_F16>, grid, dim3(256), 0, s, a);
+    default: return launch_pdl(psi_kernel<ST_BF16>, grid, dim3(256), 0, s, a);
+  }
+}
+
 cudaError_t launch_direct_d2q37(const StepArgs& a, int kind, int storage, cudaStream_t s) {
   switch (storage) {
     case ST_F32: return launch_direct2_st<ST_F32>(a, kind, sm_count(), s);

@@ -62,7 +62,8 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 enum Kind : int {
   KIND_LOCAL = 0,    // sources need only the node itself (F_i)
   KIND_THERMAL = 1,  // + H_i: theta of the 2D / 3D nearest neighbours
-  KIND_SC = 2        // + F^SC (and P_i): psi of the reach-3 neighbourhood
+  KIND_SC = 2,       // + F^SC (and P_i): psi of the reach-3 neighbourhood
+  KIND_SCF = 3       // the same with psi of this step read from a field (psi_d2q37 wrote it)
 };
 enum Storage : int { ST_F32 = 0, ST_F16 = 1, ST_BF16 = 2 };
 enum ForceMode : int { FORCE_NONE = 0, FORCE_UNIFORM = 1, FORCE_FIELD = 2, FORCE_PROFILE_Y = 3 };
@@ -109,7 +110,8 @@ struct StepArgs {
   unsigned* flags;
   unsigned long long* ms_ctr;
   // in-place (AA) step: the previous step's neighbour field (theta - 1 or psi)
-  // read on the tile's frame, and this step's written per node
+  // read on the tile's frame, and this step's written per node; KIND_SCF: psi of
+  // this step, read
   const float* aux_rd;
   float* aux_wr;
 };
@@ -161,6 +163,11 @@ cudaError_t launch_step_d2q37(const StepArgs& a, int kind, int storage, bool mom
 // straight into registers; and whether it is the faster one for a domain (tma:
 // the staged kernel could use TMA).
 bool direct_d2q37(int kind, int nx, int ny, bool tma);
+// Whether the pseudopotential step of a domain is two launches: psi of every
+// node of the state a.fin into a.aux_wr, and the direct step of KIND_SCF, which
+// reads it from a.aux_rd.
+bool two_launch_d2q37(int storage, int nx, int ny, bool tma);
+cudaError_t launch_psi_d2q37(const StepArgs& a, int storage, cudaStream_t s);
 cudaError_t launch_direct_d2q37(const StepArgs& a, int kind, int storage, cudaStream_t s);
 // tmap: {whole-row box, single-row} maps of the input buffer for the persistent
 // whole-row kernel (nx = 32, 64, 128, 256), or null.

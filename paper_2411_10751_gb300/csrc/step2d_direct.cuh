@@ -8,6 +8,9 @@
 // pitch or the periodic edge, where the staged kernel needs 16-byte aligned
 // rows for its TMA boxes and otherwise fills its planes in two to five passes
 // per thread.  The frame's lines are the neighbour tiles' (L1 or L2).
+// The pseudopotential kind also has a two-launch form (KIND_SCF): psi_kernel
+// writes psi of every node, and the step loads it on the tile and its frame, so
+// that no frame node's 37 populations are pulled and summed again.
 // Node arithmetic, tile and frame are those of the staged kernel, so the
 // results are the same bit for bit.
 #pragma once
@@ -20,7 +23,8 @@ template <int KIND>
 struct Direct2 {
   static constexpr int BX = 32, BY = 8, OWN = BX * BY;
   static constexpr int H = KIND == KIND_SC ? 3 : (KIND == KIND_THERMAL ? 1 : 0);
-  using Fr = Frame2<BX, BY, (H > 0 ? H : 1)>;
+  static constexpr int HF = KIND == KIND_SCF ? 3 : H;   // frame of the neighbour field
+  using Fr = Frame2<BX, BY, (HF > 0 ? HF : 1)>;
   static constexpr int FRAME = H > 0 ? Fr::count : 0;
   static constexpr int NT = OWN + (FRAME + 31) / 32 * 32;
 };
@@ -30,6 +34,17 @@ __device__ __forceinline__ int wrap_up(int v, int n) {
   if (v < 0) return v + n;
   if (v >= n) v -= n;
   return v < n ? v : v % n;
+}
+
+// psi of this step on the tile and its frame, from the field (KIND_SCF); the
+// caller synchronises before reading it
+template <class Fr, int HF, int NT>
+__device__ __forceinline__ void load_psi_tile(const StepArgs& a, float* aux, int x0, int y0, int tid) {
+  for (int k = tid; k < Fr::SW * Fr::SH; k += NT) {
+    const int j = k / Fr::SW, i = k - j * Fr::SW;
+    const int X = wrap_up(x0 - HF + i, a.nx), Y = wrap_up(y0 - HF + j, a.ny);
+    aux[frm<Fr>(k)] = __ldg(a.aux_rd + HLBM_IDX(Y * a.nx + X, a.N, DBG_AUX));
+  }
 }
 
 // theta or psi of a frame node, from its pulled populations
@@ -85,6 +100,7 @@ __device__ __forceinline__ void direct_tile(const StepArgs& a, float* aux, int x
   const int x = wrap_up(xr, nx), y = wrap_up(yr, ny), node = y * nx + x;
   const bool active = own && xr < nx && yr < ny;
   if (H == 0 && !own) return;
+  if constexpr (KIND == KIND_SCF) load_psi_tile<Fr, D::HF, D::OWN>(a, aux, x0, y0, tid);
   gather<L, C>(fin, a.N, nx, ny, 1, x, y, 0, g);
   if constexpr (H > 0 && BESIDE) {
     if (!own) {
@@ -99,11 +115,11 @@ __device__ __forceinline__ void direct_tile(const StepArgs& a, float* aux, int x
   float ga[3];
   accel<2>(a, node, y, ga);
   float Fx = vmul(rho, ga[0]), Fy = vmul(rho, ga[1]), sigma = 0.f;
-  const float* ap = aux + j * Fr::SW + i;
-  if constexpr (KIND == KIND_SC) {
-    const float psi = psi_of<L>(a, dr, dr_l);
-    aux[frm<Fr>(j * Fr::SW + i)] = psi;
+  const float* ap = aux + (j + D::HF - H) * Fr::SW + i + D::HF - H;
+  if constexpr (KIND == KIND_SC || KIND == KIND_SCF) {
+    if constexpr (KIND == KIND_SC) aux[frm<Fr>(j * Fr::SW + i)] = psi_of<L>(a, dr, dr_l);
     __syncthreads();
+    const float psi = ap[0];
     // F^SC = -G psi(x) sum_i w_i psi(x + c_i) c_i with G = -1
     float sx = 0.f, sy = 0.f;
     static_for<L::NPAIR>([&](auto P) {
@@ -150,7 +166,7 @@ __device__ __forceinline__ void direct_tile(const StepArgs& a, float* aux, int x
   poly2<L>(s, a.omega, a.beta, K);
   const float om1 = 1.f - a.omega;
   K[0] = vfma(-om1, acc, K[0]);
-  if constexpr (KIND == KIND_SC) K[0] = vadd(K[0], dr_l);
+  if constexpr (KIND == KIND_SC || KIND == KIND_SCF) K[0] = vadd(K[0], dr_l);
   apply_poly_h<L, 15>(g, K, om1, dr);
   const uint32_t salt = std::is_same<T, float>::value ? 0u : node_salt(node, g[0]);
   if (!HLBM_IN(node, a.N, DBG_STORE)) return;
@@ -165,7 +181,7 @@ __device__ __forceinline__ void direct_tile(const StepArgs& a, float* aux, int x
 template <int ST, int KIND, int PER>
 __global__ void __launch_bounds__(Direct2<KIND>::NT, PER) step2d_direct_kernel(const __grid_constant__ StepArgs a) {
   using D = Direct2<KIND>;
-  __shared__ float aux[D::H > 0 ? D::Fr::SW * D::Fr::SH : 1];
+  __shared__ float aux[D::HF > 0 ? D::Fr::SW * D::Fr::SH : 1];
   grid_dependency_wait();
   direct_tile<ST, KIND, D::NT>(a, aux, blockIdx.x * D::BX, blockIdx.y * D::BY);
 }
@@ -178,7 +194,7 @@ __global__ void __launch_bounds__(Direct2<KIND>::NT, PER) step2d_direct_kernel(c
 // one block per SM without spills: 64 x 64 5.0 -> 4.4 us).
 template <int KIND>
 constexpr int direct2_per_sm() {
-  return KIND == KIND_LOCAL ? 3 : 2;
+  return KIND == KIND_LOCAL || KIND == KIND_SCF ? 3 : 2;
 }
 
 template <int ST, int KIND, int PER>
@@ -192,8 +208,22 @@ cudaError_t launch_direct2_st(const StepArgs& a, int kind, int sms, cudaStream_t
   if (kind == KIND_SC)
     return (int)(grid.x * grid.y) <= sms ? launch_direct2<ST, KIND_SC, 1>(a, grid, s)
                                          : launch_direct2<ST, KIND_SC, direct2_per_sm<KIND_SC>()>(a, grid, s);
+  if (kind == KIND_SCF) return launch_direct2<ST, KIND_SCF, direct2_per_sm<KIND_SCF>()>(a, grid, s);
   if (kind == KIND_THERMAL) return launch_direct2<ST, KIND_THERMAL, direct2_per_sm<KIND_THERMAL>()>(a, grid, s);
   return launch_direct2<ST, KIND_LOCAL, direct2_per_sm<KIND_LOCAL>()>(a, grid, s);
+}
+
+// psi of every node (KIND_SCF): one node per thread, 37 loads and the density's
+// sum, so four blocks fit an SM.
+template <int ST>
+__global__ void __launch_bounds__(256, 4) psi_kernel(const __grid_constant__ StepArgs a) {
+  const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 8 + threadIdx.x / 32;
+  grid_dependency_wait();
+  if (x >= a.nx || y >= a.ny) return;
+  float g[37];
+  gather<D2Q37, Codec<ST>>(static_cast<const typename Codec<ST>::T*>(a.fin), a.N, a.nx, a.ny, 1, x, y, 0, g);
+  const int node = y * a.nx + x;
+  a.aux_wr[HLBM_IDX(node, a.N, DBG_AUX)] = frame_value<KIND_SC>(a, g, node, y);
 }
 
 }  // namespace hlbm

@@ -51,8 +51,8 @@ def _run(HLBM, c, storage, schedule, force_kind, steps):
 
 # 7 x 7 and 9 x 40: narrower than the frame; 32 x 8: one tile; 31 .. 35: the
 # remainders of a tile; 157 x 151: tiles around the SM count and odd rows;
-# 219 x 300: several waves of blocks
-SIZES = [(7, 7), (9, 40), (32, 8), (33, 9), (34, 15), (35, 17), (64, 64), (157, 151), (219, 300)]
+# 219 x 300, 288 x 290: several waves of blocks, rows off and on the 16-byte grid
+SIZES = [(7, 7), (9, 40), (32, 8), (33, 9), (34, 15), (35, 17), (64, 64), (157, 151), (219, 300), (288, 290)]
 
 
 @pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])

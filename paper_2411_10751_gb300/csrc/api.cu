@@ -1004,8 +1004,8 @@ hlbm_status hlbm_set_tile(hlbm_ctx* c, int rows, int nodes_per_thread, int persi
 hlbm_status hlbm_synchronize(hlbm_ctx* c) {
   if (!c) return HLBM_EINVAL;
   if (!c->stream) return HLBM_OK;
+  if (c->status && c->initialised) return check_status(c);   // synchronises
   HLBM_CUDA(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-  if (c->status && c->initialised) return check_status(c);
   return HLBM_OK;
 }
 
@@ -1106,13 +1106,30 @@ hlbm_status hlbm_adjoint_run(hlbm_ctx* c, int steps, int ckpt_every, void* works
       c->cur = cur0 ^ 1;
       c->steps += steps;
     } else {
-      for (int k = 0; k < nseg; ++k) {
-        HLBM_CUDA(c, cudaMemcpyAsync(state(k), c->pop[c->cur], sbytes, cudaMemcpyDeviceToDevice, c->stream),
-                  "checkpoint");
+      // a segment's last step writes its successor's checkpoint, and the steps
+      // of the last segment write the slots that the reverse sweep would
+      // otherwise recompute; the steps between alternate between the context's
+      // other buffer and the first of those slots, free until then
+      HLBM_CUDA(c, cudaMemcpyAsync(state(0), c->pop[cur0], sbytes, cudaMemcpyDeviceToDevice, c->stream), "checkpoint");
+      const void* src = state(0);
+      for (int k = 0, n = 0; k < nseg; ++k) {
+        const bool last = k == nseg - 1;
         const int len = std::min(K, steps - k * K);
-        for (int j = 0; j < len; ++j) HLBM_CUDA(c, one_step(c), "forward step");
-        c->steps += len;
+        for (int j = 0; j < len; ++j, ++n) {
+          void* dst;
+          if (j == len - 1) dst = last ? c->pop[cur0 ^ (steps & 1)] : state(k + 1);
+          else if (last) dst = state((size_t)nseg + j);
+          else dst = (j & 1) ? state(nseg) : c->pop[cur0 ^ 1];
+          StepArgs a = make_args(c);
+          a.fin = src;
+          a.fout = dst;
+          a.reverse = n & 1;
+          HLBM_CUDA(c, launch_step(c, a, false), "forward step");
+          src = dst;
+        }
       }
+      c->cur = cur0 ^ (steps & 1);
+      c->steps += steps;
     }
   }
   // seed from the final state: lambda_T, dL/dg at T, kinetic energy
@@ -1151,7 +1168,7 @@ hlbm_status hlbm_adjoint_run(hlbm_ctx* c, int steps, int ckpt_every, void* works
     const int len = std::min(K, steps - k * K);
     // states of the segment: j = 0 is checkpoint k, j >= 1 are recomputed into slots nseg + j - 1
     auto seg = [&](int j) { return j == 0 ? (K == 1 ? slot(k) : state(k)) : state((size_t)nseg + j - 1); };
-    for (int j = 1; j < len; ++j) {
+    for (int j = 1; j < len && k < nseg - 1; ++j) {   // (the forward sweep kept the last segment's)
       StepArgs a = make_args(c);   // staged by tensor maps of the workspace slots
       a.fin = seg(j - 1);
       a.fout = seg(j);

@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(kBX * kBY / NPT, 2 * NPT) aa_step_kernel(const
     nodek[k] = yck[k] * nx + xc;
   }
 
+  grid_dependency_wait();
   // the previous step's neighbour field, on the tile and its frame
   if constexpr (H > 0) {
     for (int k = tid; k < SW * SH; k += NT) {
@@ -306,8 +307,8 @@ cudaError_t launch_kind(const StepArgs& a, bool odd, bool mom, cudaStream_t s) {
     else aa_step_kernel<ST, KIND, false, true, 1><<<grid, block, 0, s>>>(a);
   } else {
     const dim3 block(kBX, kBY / 2);
-    if (odd) aa_step_kernel<ST, KIND, true, false, 2><<<grid, block, 0, s>>>(a);
-    else aa_step_kernel<ST, KIND, false, false, 2><<<grid, block, 0, s>>>(a);
+    return odd ? launch_pdl(aa_step_kernel<ST, KIND, true, false, 2>, grid, block, 0, s, a)
+               : launch_pdl(aa_step_kernel<ST, KIND, false, false, 2>, grid, block, 0, s, a);
   }
   return cudaGetLastError();
 }

@@ -428,6 +428,7 @@ __global__ void __launch_bounds__(256, 2)
     s_next[slot] = t;
     if (t < ntiles) mbar_arrive_expect_tx(bar, S::TX);
   };
+  grid_dependency_wait();
   if (tid == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
@@ -508,7 +509,8 @@ cudaError_t launch_adj_step(const AdjArgs& a, const CUtensorMap* tm, cudaStream_
   if (tm && a.ctr && adj_rows_eligible<ST>(a)) {
     const int tiles = ((a.ny + kAdjRowNodes / a.nx - 1) / (kAdjRowNodes / a.nx)) * a.nz;
     const int ctas = std::min(tiles, adj_rows_ctas<ST>());
-    adjoint_rows_kernel<ST><<<ctas, 256, AdjRowsSmem<ST>::BYTES, s>>>(a, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5]);
+    return launch_pdl(adjoint_rows_kernel<ST>, dim3(ctas), dim3(256), AdjRowsSmem<ST>::BYTES, s, a, tm[0], tm[1], tm[2],
+                      tm[3], tm[4], tm[5]);
   } else {
     adjoint_step_kernel<D3Q39, ST><<<(unsigned)((a.N + 127) / 128), 128, 0, s>>>(a);
   }

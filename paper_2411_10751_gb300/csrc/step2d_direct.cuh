@@ -29,13 +29,6 @@ struct Direct2 {
   static constexpr int NT = OWN + (FRAME + 31) / 32 * 32;
 };
 
-// v mod n for v >= -n
-__device__ __forceinline__ int wrap_up(int v, int n) {
-  if (v < 0) return v + n;
-  if (v >= n) v -= n;
-  return v < n ? v : v % n;
-}
-
 // psi of this step on the tile and its frame, from the field (KIND_SCF); the
 // caller synchronises before reading it
 template <class Fr, int HF, int NT>

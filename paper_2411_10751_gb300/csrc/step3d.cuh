@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(32 * BY / NPT, (min_ctas3<MOM, NPT>()))
   constexpr float inv_c0 = (float)(1.0 / L::c0);
   __shared__ double red[MOM ? (NT / 32) * 6 : 1];
 
+  grid_dependency_wait();
   const T* __restrict__ fin = static_cast<const T*>(a.fin);
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
@@ -235,6 +236,7 @@ __global__ void __launch_bounds__(128, 3)
     s_next[slot] = t;
     if (t < ntiles) mbar_arrive_expect_tx(bar, tx);
   };
+  grid_dependency_wait();
   if (tid == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
@@ -366,15 +368,14 @@ cudaError_t launch_step3d_st(const StepArgs& a, int kind, bool mom, int rows, in
     const int by = kRows3Nodes / a.nx;
     const int tiles = ((a.ny + by - 1) / by) * a.nz;
     const int ctas = std::min(tiles, rows3_ctas<ST>());
-    step3d_rows_kernel<ST><<<ctas, 128, rows3_smem<ST>(), s>>>(a, tmaps[0], tmaps[1], tmaps[2]);
-    return cudaGetLastError();
+    return launch_pdl(step3d_rows_kernel<ST>, dim3(ctas), dim3(128), rows3_smem<ST>(), s, a, tmaps[0], tmaps[1], tmaps[2]);
   }
   const int by = (rows == 4) ? 4 : 8;
   const dim3 grid((a.nx + 31) / 32, (a.ny + by - 1) / by, a.nz);
   if (mom) step3d_kernel<ST, true, 8, 1><<<dim3((a.nx + 31) / 32, (a.ny + 7) / 8, a.nz), dim3(32, 8), 0, s>>>(a);
-  else if (by == 4) step3d_kernel<ST, false, 4, 1><<<grid, dim3(32, 4), 0, s>>>(a);
-  else if (npt == 2) step3d_kernel<ST, false, 8, 2><<<grid, dim3(32, 4), 0, s>>>(a);
-  else step3d_kernel<ST, false, 8, 1><<<grid, dim3(32, 8), 0, s>>>(a);
+  else if (by == 4) return launch_pdl(step3d_kernel<ST, false, 4, 1>, grid, dim3(32, 4), 0, s, a);
+  else if (npt == 2) return launch_pdl(step3d_kernel<ST, false, 8, 2>, grid, dim3(32, 4), 0, s, a);
+  else return launch_pdl(step3d_kernel<ST, false, 8, 1>, grid, dim3(32, 8), 0, s, a);
   return cudaGetLastError();
 }
 

@@ -258,6 +258,13 @@ __device__ __forceinline__ int wrapm(int v, int n) {
   return v < 0 ? v + n : v;
 }
 
+// v mod n for v >= -n
+__device__ __forceinline__ int wrap_up(int v, int n) {
+  if (v < 0) return v + n;
+  if (v >= n) v -= n;
+  return v < n ? v : v % n;
+}
+
 // ------------------------------------------------------------------ gather
 // g_i(x) = stored_i(x - c_i), periodic.  x in [0,nx), y in [0,ny), z in [0,nz).
 template <class L, class C>

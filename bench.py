@@ -55,7 +55,7 @@ WORKLOADS = {
     "tg3d256": (lambda: W.taylor_green_3d(n=256), "D3Q39 compressible Taylor-Green 256^3, Ma=0.3, tau=0.6, body force"),
     "droplet512": (lambda: W.droplet(n=512), "D2Q37 vdW droplet 512x512 (T/Tc 0.85, k 0.01, r0 N/4), tau=0.8"),
     "droplet1024": (lambda: W.droplet(n=1024), "D2Q37 vdW droplet 1024x1024 (T/Tc 0.85, k 0.01, r0 N/4), tau=0.8"),
-    # wall-bounded step (Tamm-Mott-Smith walls, two launches per step) and the
+    # wall-bounded step (Tamm-Mott-Smith walls, three launches per step) and the
     # Carnahan-Starling pseudopotential
     "rb1024": (lambda: W.rayleigh_benard(nx=1024, ny=1026, Ra=10000.0, roll=0.01),
                "D2Q37 Rayleigh-Benard, 1024x1026 between two walls (Ra 1e4, Pr 1.41, theta 1.4 / 1.0)"),
@@ -134,7 +134,7 @@ def _launches(case, sched, steps) -> int:
     """Step-kernel launches of hlbm_step(steps): one per step, or one per
     block of up to 1024 steps for the multi-step kernel."""
     if case.params.get("walls"):
-        return 3 * steps   # wall completion, moments, collision
+        return 3 * steps   # the rows next to the lower and the upper wall, the rows between
     if not _multistep(case, sched):
         return steps
     tiles = (case.nx // 32) * (case.ny // sched[0])

@@ -282,7 +282,7 @@ __device__ __forceinline__ void gather(const typename C::T* __restrict__ f, long
     constexpr int cx = L::c(i, 0), cy = L::c(i, 1), cz = L::c(i, 2);
     int off = ys[cy + 3] + xs[cx + 3];
     if constexpr (L::D == 3) off += zs[cz + 3];
-    g[i] = C::ld(f + HLBM_IDX((size_t)i * (size_t)N + off, (long long)L::Q * N, DBG_GATHER));
+    g[i] = C::ld(f + (size_t)i * (size_t)N + (unsigned)HLBM_IDX(off, N, DBG_GATHER));
   });
 }
 

@@ -631,10 +631,7 @@ __global__ void __launch_bounds__(wall_threads<THERMAL>(), THERMAL ? 2 : 3)
   float g[37];
   WallMoments m;
   if (needed) {
-    static_for<37>([&](auto I) {
-      constexpr int q = I;
-      g[q] = ldpop<ST>(a, q, wrapx(x - L::c(q, 0), nx), y - L::c(q, 1));
-    });
+    gather<L, Codec<ST>>(static_cast<const typename Codec<ST>::T*>(a.fin), a.N, nx, a.ny, 1, x, y, 0, g);
     m = wall_moments(a, g, node, y);
     if constexpr (THERMAL) tbs[j * SW + i] = m.tb;
   }

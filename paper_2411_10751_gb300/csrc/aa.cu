@@ -24,7 +24,7 @@
 // written) + about 4 (the staged field, neighbours served by L2): 304 B FP32.
 #include "internal.h"
 #include "lattice.cuh"
-#include "step_common.cuh"
+#include "step2d.cuh"
 
 #include <type_traits>
 
@@ -41,23 +41,27 @@ constexpr int frame_of() {
   return KIND == KIND_SC ? 3 : (KIND == KIND_THERMAL ? 1 : 0);
 }
 
-// ODD: the step's parity; MOM: moments readout (no store).  NPT nodes per
-// thread: lane k of thread (tx, ty) is tile row ty + k kBY / NPT, and with
-// NPT = 2 the node arithmetic runs on paired FP32 lanes (float2), rounding
-// exactly like the one-node form.
-template <int ST, int KIND, bool ODD, bool MOM, int NPT>
-__global__ void __launch_bounds__(kBX * kBY / NPT, 2 * NPT) aa_step_kernel(const __grid_constant__ StepArgs a) {
+// One tile of the step.  ODD: the step's parity; MOM: moments readout (no
+// store).  NPT nodes per thread: lane k of thread (tx, ty) is tile row
+// ty + k kBY / NPT, and with NPT = 2 the node arithmetic runs on paired FP32
+// lanes (float2), rounding exactly like the one-node form.
+// aux: the neighbour field on the tile and its frame (shared memory).  sp: null,
+// or the tile's populations staged by TMA as Cfg2<ST, KIND_LOCAL> lays them out
+// (population i of the tile shifted by -c_i on odd steps); ready() returns once
+// they have landed, and staged_done() is called after a barrier once they are
+// all in registers.
+template <int ST, int KIND, bool ODD, bool MOM, int NPT, class Ready, class Done>
+__device__ __forceinline__ void aa_tile(const StepArgs& a, float* aux, const typename Codec<ST>::T* sp, int x0, int y0,
+                                        Ready&& ready, Done&& staged_done) {
   using T = typename Codec<ST>::T;
   using V = typename std::conditional<NPT == 2, float2, float>::type;
+  using Cf = Cfg2<ST, KIND_LOCAL, false, kBY>;
   constexpr int H = frame_of<KIND>();
   constexpr int SW = kBX + 2 * H, SH = kBY + 2 * H;
   constexpr int TR = kBY / NPT, NT = kBX * TR;   // thread rows, threads
-  __shared__ float aux[(H > 0) ? SW * SH : 1];
-  __shared__ double red[TR][6];
   const int nx = a.nx, ny = a.ny;
   const size_t N = (size_t)a.N;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kBX + tx;
-  const int x0 = blockIdx.x * kBX, y0 = blockIdx.y * kBY;
   const int x = x0 + tx;
   const int xc = x < nx ? x : x % nx;   // inactive lanes still compute (the frame is shared)
   int yck[NPT], nodek[NPT];
@@ -70,7 +74,6 @@ __global__ void __launch_bounds__(kBX * kBY / NPT, 2 * NPT) aa_step_kernel(const
     nodek[k] = yck[k] * nx + xc;
   }
 
-  grid_dependency_wait();
   // the previous step's neighbour field, on the tile and its frame
   if constexpr (H > 0) {
     for (int k = tid; k < SW * SH; k += NT) {
@@ -78,12 +81,23 @@ __global__ void __launch_bounds__(kBX * kBY / NPT, 2 * NPT) aa_step_kernel(const
       const int X = wrapm(x0 - H + i, nx), Y = wrapm(y0 - H + j, ny);
       aux[k] = __ldg(a.aux_rd + HLBM_IDX((long long)Y * nx + X, a.N, DBG_AUX));
     }
-    __syncthreads();
   }
+  ready();
+  if (H > 0 || sp) __syncthreads();
 
   // the nodes' populations at time t
   const T* __restrict__ f = static_cast<const T*>(a.fin);
   V g[37];
+  if (sp) {
+    static_for<37>([&](auto I) {
+      constexpr int i = I;
+#pragma unroll
+      for (int k = 0; k < NPT; ++k)
+        set_lane(g[i], k, to_float(sp[stg<Cf>(i, (ty + k * TR) * Cf::WB + tx + (ODD ? Cf::rem(i) : 0))]));
+    });
+    __syncthreads();
+    staged_done();
+  } else {
   int xs[7], ys[NPT][7];
 #pragma unroll
   for (int d = -3; d <= 3; ++d) {
@@ -103,6 +117,8 @@ __global__ void __launch_bounds__(kBX * kBY / NPT, 2 * NPT) aa_step_kernel(const
       }
     }
   });
+  staged_done();
+  }
 
   V dr, dr_l, acc, J[3], Pih;
   moments_h<L>(g, dr, dr_l, acc, J, Pih);
@@ -173,6 +189,7 @@ __global__ void __launch_bounds__(kBX * kBY / NPT, 2 * NPT) aa_step_kernel(const
       v[5] += bad ? 1.0 : 0.0;
     }
     if (a.partials) {
+      __shared__ double red[TR][6];
 #pragma unroll
       for (int k = 0; k < 6; ++k)
         for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
@@ -263,6 +280,121 @@ __global__ void __launch_bounds__(kBX * kBY / NPT, 2 * NPT) aa_step_kernel(const
   }
 }
 
+template <int ST, int KIND, bool ODD, bool MOM, int NPT>
+__global__ void __launch_bounds__(kBX * kBY / NPT, 2 * NPT) aa_step_kernel(const __grid_constant__ StepArgs a) {
+  constexpr int H = frame_of<KIND>();
+  __shared__ float aux[(H > 0) ? (kBX + 2 * H) * (kBY + 2 * H) : 1];
+  grid_dependency_wait();
+  aa_tile<ST, KIND, ODD, MOM, NPT>(a, aux, nullptr, blockIdx.x * kBX, blockIdx.y * kBY, [] {}, [] {});
+}
+
+// Persistent CTAs, two nodes per thread, that stage the next tile's populations
+// by TMA while the current one collides (tiles in row-major order from the
+// step's never-reset counter, backwards on every other step; tiles whose boxes
+// would cross the periodic edge pull as above).  A tile writes only the slots it
+// read, so the copies of the next tile wait for nothing; what a box holds beyond
+// its tile's slots may be changing meanwhile and is not used.
+template <int ST, int KIND>
+struct AaRing {
+  using Cf = Cfg2<ST, KIND_LOCAL, false, kBY>;
+  static constexpr int H = frame_of<KIND>();
+  static constexpr int AUX = H > 0 ? ((kBX + 2 * H) * (kBY + 2 * H) * 4 + 127) / 128 * 128 : 0;
+  static constexpr int BYTES = Cf::POP_BYTES + AUX + 128;
+};
+
+template <int ST, int KIND, bool ODD>
+__global__ void __launch_bounds__(kBX * kBY / 2, 4)
+    aa_persistent_kernel(const __grid_constant__ StepArgs a, const __grid_constant__ CUtensorMap tmap) {
+  using R = AaRing<ST, KIND>;
+  using Cf = typename R::Cf;
+  using T = typename Codec<ST>::T;
+  constexpr int W = kBY / 2;   // warps
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ int s_first, s_ahead;
+  T* sp = reinterpret_cast<T*>(smem);
+  float* aux = reinterpret_cast<float*>(smem + Cf::POP_BYTES);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + Cf::POP_BYTES + R::AUX);
+  const int tid = threadIdx.y * kBX + threadIdx.x, warp = threadIdx.y;
+  const int ntx = (a.nx + kBX - 1) / kBX, ntiles = ntx * ((a.ny + kBY - 1) / kBY);
+  const unsigned long long period = (unsigned long long)ntiles + gridDim.x;
+  if (!HLBM_IN(smem_u32(smem) & 127u, 1, DBG_SMEM)) return;   // TMA destinations need 128-byte alignment
+  auto origin = [&](int t, int& x0, int& y0) {
+    const int u = a.reverse ? ntiles - 1 - t : t;
+    const int ty = u / ntx;
+    y0 = ty * kBY;
+    x0 = (u - ty * ntx) * kBX;
+  };
+  auto stage = [&](int t) {   // lane 0 of every warp: a share of the planes of tile t
+    if (t >= ntiles) return;
+    int x0, y0;
+    origin(t, x0, y0);
+    if (!tile_boxed<Cf>(a, x0, y0)) return;
+    fence_proxy_async_smem();
+    if (warp == 0) mbar_arrive_expect_tx(bar, Cf::TX_BYTES);
+    static_for<37>([&](auto I) {
+      constexpr int i = I;
+      if (i % W != warp) return;
+      const int bx = ODD ? x0 - L::c(i, 0) - Cf::rem(i) : x0, by = ODD ? y0 - L::c(i, 1) : y0;
+      if (!HLBM_IN(bx % Cf::A, 1, DBG_BOX) || !HLBM_IN(bx, a.nx - Cf::WB + 1, DBG_BOX) ||
+          !HLBM_IN(by, a.ny - Cf::HB + 1, DBG_BOX))
+        return;   // (debug build) a dropped copy leaves the barrier short
+      tma_load_3d(sp + i * Cf::PLANE, &tmap, bx, by, ODD ? aa_opp(i) : i, bar);
+    });
+  };
+  unsigned long long raw = 0;
+  grid_dependency_wait();
+  if (tid == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+    const int t0 = (int)(atomicAdd(a.tile_ctr, 1ull) % period);
+    s_first = t0;
+    s_ahead = t0 < ntiles ? (int)(atomicAdd(a.tile_ctr, 1ull) % period) : t0;
+  }
+  __syncthreads();
+  int t = s_first;
+  if ((tid & 31) == 0) stage(t);
+  uint32_t phase = 0;
+  while (t < ntiles) {
+    const int tn = s_ahead;
+    int x0, y0;
+    origin(t, x0, y0);
+    const bool boxed = tile_boxed<Cf>(a, x0, y0);
+    if (boxed) {
+      const bool ok = mbar_wait_bounded(bar, phase, a.wait_ns);
+      if (!__syncthreads_and(ok)) {
+        if (tid == 0) atomicExch(a.status, (int)5 /* HLBM_ETIMEOUT */);
+        mbar_wait_bounded(bar, phase, a.wait_ns);
+        __syncthreads();
+        return;
+      }
+      phase ^= 1u;
+    }
+    aa_tile<ST, KIND, ODD, false, 2>(a, aux, boxed ? sp : nullptr, x0, y0, [] {}, [&] {
+      if ((tid & 31) == 0) stage(tn);
+      if (tid == 0 && tn < ntiles) raw = atomicAdd(a.tile_ctr, 1ull);
+    });
+    __syncthreads();   // every thread has read s_ahead and is done with aux
+    if (tid == 0) s_ahead = tn < ntiles ? (int)(raw % period) : tn;
+    __syncthreads();
+    t = tn;
+  }
+}
+
+template <int ST, int KIND>
+int aa_persistent_ctas() {
+  static std::atomic<int> cache[kMaxDevicesCached];
+  return per_device_cached(cache, [](int dev) {
+    int sms = 0, e = 0, o = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaFuncSetAttribute(aa_persistent_kernel<ST, KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AaRing<ST, KIND>::BYTES);
+    cudaFuncSetAttribute(aa_persistent_kernel<ST, KIND, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AaRing<ST, KIND>::BYTES);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&e, aa_persistent_kernel<ST, KIND, false>, kBX * kBY / 2, AaRing<ST, KIND>::BYTES);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, aa_persistent_kernel<ST, KIND, true>, kBX * kBY / 2, AaRing<ST, KIND>::BYTES);
+    const int per = std::min(e, o);   // one grid for both parities: they share the counter's period
+    return (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
+  });
+}
+
 // Initial state in the even layout: slot i of node x = f^eq_i(x); the
 // neighbour field the first step reads (theta - 1, or psi of the density).
 template <int ST, int KIND>
@@ -299,7 +431,7 @@ __global__ void __launch_bounds__(256) aa_init_kernel(const __grid_constant__ St
 
 // steps: two nodes per thread (paired FP32 lanes); the moments readout: one
 template <int ST, int KIND>
-cudaError_t launch_kind(const StepArgs& a, bool odd, bool mom, cudaStream_t s) {
+cudaError_t launch_kind(const StepArgs& a, bool odd, bool mom, const CUtensorMap* tmap, cudaStream_t s) {
   const dim3 grid((a.nx + kBX - 1) / kBX, (a.ny + kBY - 1) / kBY);
   if (mom) {
     const dim3 block(kBX, kBY);
@@ -307,6 +439,11 @@ cudaError_t launch_kind(const StepArgs& a, bool odd, bool mom, cudaStream_t s) {
     else aa_step_kernel<ST, KIND, false, true, 1><<<grid, block, 0, s>>>(a);
   } else {
     const dim3 block(kBX, kBY / 2);
+    if (tmap) {
+      const dim3 ctas(std::min((int)(grid.x * grid.y), aa_persistent_ctas<ST, KIND>()));
+      return odd ? launch_pdl(aa_persistent_kernel<ST, KIND, true>, ctas, block, AaRing<ST, KIND>::BYTES, s, a, *tmap)
+                 : launch_pdl(aa_persistent_kernel<ST, KIND, false>, ctas, block, AaRing<ST, KIND>::BYTES, s, a, *tmap);
+    }
     return odd ? launch_pdl(aa_step_kernel<ST, KIND, true, false, 2>, grid, block, 0, s, a)
                : launch_pdl(aa_step_kernel<ST, KIND, false, false, 2>, grid, block, 0, s, a);
   }
@@ -314,10 +451,10 @@ cudaError_t launch_kind(const StepArgs& a, bool odd, bool mom, cudaStream_t s) {
 }
 
 template <int ST>
-cudaError_t launch_st(const StepArgs& a, int kind, bool odd, bool mom, cudaStream_t s) {
-  if (kind == KIND_SC) return launch_kind<ST, KIND_SC>(a, odd, mom, s);
-  if (kind == KIND_THERMAL) return launch_kind<ST, KIND_THERMAL>(a, odd, mom, s);
-  return launch_kind<ST, KIND_LOCAL>(a, odd, mom, s);
+cudaError_t launch_st(const StepArgs& a, int kind, bool odd, bool mom, const CUtensorMap* tmap, cudaStream_t s) {
+  if (kind == KIND_SC) return launch_kind<ST, KIND_SC>(a, odd, mom, tmap, s);
+  if (kind == KIND_THERMAL) return launch_kind<ST, KIND_THERMAL>(a, odd, mom, tmap, s);
+  return launch_kind<ST, KIND_LOCAL>(a, odd, mom, tmap, s);
 }
 
 template <int ST>
@@ -332,11 +469,12 @@ cudaError_t init_st(const StepArgs& a, int kind, const float* rho, const float* 
 
 }  // namespace
 
-cudaError_t launch_aa(const StepArgs& a, int kind, int storage, bool odd, bool mom, cudaStream_t s) {
+cudaError_t launch_aa(const StepArgs& a, int kind, int storage, bool odd, bool mom, const CUtensorMap* tmap,
+                      cudaStream_t s) {
   switch (storage) {
-    case ST_F32: return launch_st<ST_F32>(a, kind, odd, mom, s);
-    case ST_F16: return launch_st<ST_F16>(a, kind, odd, mom, s);
-    default: return launch_st<ST_BF16>(a, kind, odd, mom, s);
+    case ST_F32: return launch_st<ST_F32>(a, kind, odd, mom, tmap, s);
+    case ST_F16: return launch_st<ST_F16>(a, kind, odd, mom, tmap, s);
+    default: return launch_st<ST_BF16>(a, kind, odd, mom, tmap, s);
   }
 }
 

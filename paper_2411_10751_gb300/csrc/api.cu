@@ -512,6 +512,16 @@ cudaError_t wall_step(hlbm_ctx* c) {
   return e;
 }
 
+// Whether the in-place step runs its persistent TMA-staged form: FP32, from the
+// size on where its one buffer streams from HBM (us per step, pulls / staged:
+// body force 1024 x 1024 55.6 / 50.8, thermal 63.4 / 56.8, pseudopotential 73.1 /
+// 64.5; 2048 x 2048 208.9 / 199.1, 240.2 / 214.3, 272.4 / 239.4; inside L2, 512 x 512,
+// 10.8 / 15.6, 12.9 / 17.9, 15.8 / 20.4).  In 16 bits the pulls are as fast or
+// faster (1024 x 1024 37.0 / 46.3, 47.9 / 52.9, 59.8 / 64.2).
+bool aa_staged(const hlbm_ctx* c) {
+  return c->tma_ok && !c->debug_skip_tma && c->storage == ST_F32 && (double)c->Q * (double)c->N * 4.0 >= 96e6;
+}
+
 // One in-place step of parity cur: reads aux[cur ^ 1], writes aux[cur].
 cudaError_t aa_step(hlbm_ctx* c, bool mom, StepArgs* margs = nullptr) {
   StepArgs a = margs ? *margs : make_args(c);
@@ -519,7 +529,14 @@ cudaError_t aa_step(hlbm_ctx* c, bool mom, StepArgs* margs = nullptr) {
   a.fout = c->pop[0];
   a.aux_rd = c->aux[c->cur ^ 1];
   a.aux_wr = c->aux[c->cur];
-  cudaError_t e = launch_aa(a, c->kind, c->storage, c->cur == 1, mom, c->stream);
+  a.reverse = c->cur;
+  const CUtensorMap* tm = nullptr;
+  if (!mom && aa_staged(c)) {
+    int wb = 0, hb = 0, ob = 0;
+    step_box_d2q37(KIND_LOCAL, c->storage, false, 8, &wb, &hb, &ob);
+    tm = tensor_map_at(c, c->pop[0], wb, hb);
+  }
+  cudaError_t e = launch_aa(a, c->kind, c->storage, c->cur == 1, mom, tm, c->stream);
   if (!mom) c->cur ^= 1;
   return e;
 }

@@ -189,7 +189,10 @@ int moment_blocks(int lattice, int nx, int ny, int nz);
 // population buffer); mom = moments readout (rho_out / u_out / theta_out,
 // partials) of the state before that step.  aa_init writes the even layout
 // and the first step's neighbour field (a.aux_wr).
-cudaError_t launch_aa(const StepArgs& a, int kind, int storage, bool odd, bool mom, cudaStream_t s);
+// tmap: map of the buffer with the boxes of step_box_d2q37(KIND_LOCAL, 8 rows) for
+// the persistent form (D2Q37 tiles staged by TMA), or null.
+cudaError_t launch_aa(const StepArgs& a, int kind, int storage, bool odd, bool mom, const CUtensorMap* tmap,
+                      cudaStream_t s);
 cudaError_t launch_aa_init(const StepArgs& a, int kind, int storage, const float* rho, const float* u,
                            const float* theta, cudaStream_t s);
 

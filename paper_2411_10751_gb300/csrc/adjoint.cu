@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(128) adjoint_step_kernel(const __grid_constant
     static_for<L::Q>([&](auto I) {
       constexpr int i = I;
       const int off = zs[L::c(i, 2) + 3] + ys[L::c(i, 1) + 3] + xs[L::c(i, 0) + 3];
-      mu[i] = __ldg(a.lam_in + (size_t)i * a.N + off);
+      mu[i] = __ldg(a.lam_in + (size_t)i * (size_t)a.N + (unsigned)off);
     });
   }
   float dg[3];

@@ -275,7 +275,7 @@ void drop_graphs(hlbm_ctx* c) {
 // block scheduling is faster.  us per step, one CTA per tile against
 // persistent, FP32 unless stated: thermal 512 x 512 (78 MB) 16.7 / 18.0, 576 x 576
 // (98 MB) 21.4 / 19.6, 1024 x 1024 60.9 / 54.9; pseudopotential 576 x 576 35.9 /
-// 34.8, 1024 x 1024 95.5 / 89.4; D3Q39 64^3 (82 MB) 14.3 / 15.0, 128^3 136.2 / 98.8,
+// 34.8, 1024 x 1024 95.5 / 89.4; D3Q39 64^3 (82 MB) 12.3 / 15.0, 128^3 136.2 / 98.8,
 // 128^3 FP16 97.1 / 79.9.  Not for D2Q37 in 16 bits, whose persistent form has 3
 // CTAs per SM instead of 4 (thermal 1024 x 1024 45.4 / 48.8), nor for the body
 // force alone, which gains at some sizes (1024 x 1024 54.1 / 53.1) and loses at

@@ -11,9 +11,10 @@
 // kind before them on all.  The pseudopotential tiles, the slowest, come first
 // in the work list, so the launch ends on short tiles.  Item and step arguments
 // are read from device memory one item ahead, by the last warps while the
-// others collide.  It is bound by instruction issue (53% of the slots) and the
-// loads' latency at 22 warps per SM: 256 domains, 6.4 M nodes, FP32, 770 -> 564 us
-// a step (the staged form spent 62 warp instructions per node, this one 45).
+// others collide.  It is bound by instruction issue (half of the slots) and the
+// loads' latency at 22 warps per SM: 256 domains, 6.4 M nodes, FP32, 770 us a step
+// staged, 564 us pulled, 515 us with 32-bit offsets in the pulls.  Three CTAs per
+// SM at 56 registers took 643 us.
 #include <algorithm>
 #include <cstdio>
 #include <cstring>

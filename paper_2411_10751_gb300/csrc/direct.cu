@@ -22,7 +22,10 @@ int sm_count() {
 // once, where the latency of a step counts (64 x 64: 4.3 -> 3.0, 5.2 -> 3.5, 8.1
 // -> 4.4; 256 x 256: 5.5 -> 4.9, 6.7 -> 5.7, 10.1 -> 8.3), and slower beyond
 // (384 x 384 body force 7.2 against 8.0, 320 x 320 thermal 7.5 against 8.3,
-// 448 x 448 pseudopotential FP16 20.1 against 24.1).
+// 448 x 448 pseudopotential FP16 20.1 against 24.1).  Both sides as of the same
+// build; with 32-bit offsets in the pulls the direct side has since gained 5 to
+// 20% (64 x 64 body force 2.7, 901 x 899 thermal FP16 46.5, pseudopotential 77.7 /
+// 63.0).
 bool direct_d2q37(int kind, int nx, int ny, bool tma) {
   if (!tma) return true;
   const long long tiles = (long long)((nx + 31) / 32) * ((ny + 7) / 8);
@@ -38,7 +41,9 @@ bool direct_d2q37(int kind, int nx, int ny, bool tma) {
 // (FP32 us per step, one launch / two: 320 x 320 15.1 / 11.5, 512 x 512 27.4 /
 // 23.8, 544 x 544 30.2 / 27.3, 640 x 640 37.8 / 39.2; 641 x 639 46.3 / 41.3, 901 x
 // 899 85.3 / 83.5, 1201 x 1199 146.3 / 139.1, FP16 133.9 / 124.4).  Aligned 16-bit
-// domains gain nothing (384 x 384 14.3 / 15.0, 512 x 512 23.1 / 23.5).
+// domains gain nothing (384 x 384 14.3 / 15.0, 512 x 512 23.1 / 23.5).  (Both
+// sides of the same build; with 32-bit offsets in the pulls two launches take
+// 37.2 at 641 x 639, 77.7 at 901 x 899.)
 bool two_launch_d2q37(int storage, int nx, int ny, bool tma) {
   if (direct_d2q37(KIND_SC, nx, ny, true)) return false;   // one wave: a launch more costs more
   return !tma || (storage == ST_F32 && 2.0 * 37 * 4 * (double)nx * ny < 96e6);

@@ -587,8 +587,8 @@ __global__ void __launch_bounds__(kEdgeThreads) wall_edge_kernel(const __grid_co
 // nodes, one thread each, whose populations stay in registers; with H_i, three
 // more warps pull the 80 nodes of the 4-neighbour ring around them for theta
 // alone (their lines are the neighbour blocks', in L1 or L2), so the
-// populations are read from memory once per step (two passes, a moments launch
-// and a collide launch, took 33 + 57 us at 1024 x 1026; this one takes 72 us).
+// populations are read from memory once per step (at 1024 x 1026 a moments and a
+// collide launch took 33 + 57 us; a whole step takes 72.7 us).
 template <bool THERMAL>
 constexpr int wall_threads() {
   return kBX * kBY + (THERMAL ? 96 : 0);

@@ -110,10 +110,10 @@ __device__ __forceinline__ void aa_tile(const StepArgs& a, float* aux, const typ
 #pragma unroll
     for (int k = 0; k < NPT; ++k) {
       if constexpr (!ODD) {
-        set_lane(g[i], k, to_float(f[HLBM_IDX((long long)i * N + nodek[k], 37 * a.N, DBG_GATHER)]));
+        set_lane(g[i], k, to_float((f + (size_t)i * N)[(unsigned)HLBM_IDX(nodek[k], a.N, DBG_GATHER)]));
       } else {
         constexpr int cx = L::c(i, 0), cy = L::c(i, 1), b = aa_opp(i);
-        set_lane(g[i], k, to_float(f[HLBM_IDX((long long)b * N + ys[k][cy + 3] + xs[cx + 3], 37 * a.N, DBG_GATHER)]));
+        set_lane(g[i], k, to_float((f + (size_t)b * N)[(unsigned)HLBM_IDX(ys[k][cy + 3] + xs[cx + 3], a.N, DBG_GATHER)]));
       }
     }
   });

@@ -60,9 +60,7 @@ struct hlbm_ctx {
   // fields: aux[cur ^ 1] is read by the next step, aux[cur] written
   bool aa = false;
   float* aux[2] = {nullptr, nullptr};
-  float* comp[2] = {nullptr, nullptr};   // walls: completed unknowns of the six wall rows of pop[0], pop[1]
-  cudaStream_t wall_stream[2] = {nullptr, nullptr};          // walls: the lower and upper edge launches
-  cudaEvent_t wall_ev[3] = {nullptr, nullptr, nullptr};      // walls: their joins, and the fork
+  float* comp = nullptr;          // walls: completed unknowns of the six wall rows
 
   bool failed = false;
   std::string msg;
@@ -127,10 +125,10 @@ Layout layout(int lattice, int nx, int ny, int nz, const hlbm_source_params* p) 
   L.off_aux = L.off_mom + 2 * L.mom_bytes;
   // in place: two neighbour fields; pseudopotential on two buffers: psi
   L.aux_bytes = (p->flags & (HLBM_AA | HLBM_SRC_SC)) ? align256((size_t)N * 4) : 0;
-  // walls: the completed unknowns of the six wall rows of each buffer, [6][37][nx] FP32
+  // walls: the completed unknowns of the six wall rows, [6][37][nx] FP32
   L.off_comp = L.off_aux + ((p->flags & HLBM_AA) ? 2 : 1) * L.aux_bytes;
   L.comp_bytes = (p->flags & HLBM_WALLS) ? align256((size_t)6 * 37 * (size_t)nx * 4) : 0;
-  L.total = L.off_comp + 2 * L.comp_bytes;
+  L.total = L.off_comp + L.comp_bytes;
   return L;
 }
 
@@ -249,8 +247,7 @@ void carve(hlbm_ctx* c) {
   c->mom[1] = L.mom_bytes ? reinterpret_cast<float*>(c->arena + L.off_mom + L.mom_bytes) : nullptr;
   c->aux[0] = L.aux_bytes ? reinterpret_cast<float*>(c->arena + L.off_aux) : nullptr;
   c->aux[1] = L.aux_bytes ? reinterpret_cast<float*>(c->arena + L.off_aux + L.aux_bytes) : nullptr;
-  c->comp[0] = L.comp_bytes ? reinterpret_cast<float*>(c->arena + L.off_comp) : nullptr;
-  c->comp[1] = L.comp_bytes ? reinterpret_cast<float*>(c->arena + L.off_comp + L.comp_bytes) : nullptr;
+  c->comp = L.comp_bytes ? reinterpret_cast<float*>(c->arena + L.off_comp) : nullptr;
 }
 
 hlbm_status ensure_stream(hlbm_ctx* c) {
@@ -458,56 +455,19 @@ WallArgs make_wall_args(const hlbm_ctx* c) {
   w.e_ref = (float)(c->p.rho0 * 2.0 * D2Q37::cs2 * tbr);
   w.mprev = c->mom[c->cur];
   w.fin = c->pop[c->cur];
-  w.comp = c->comp[c->cur];
+  w.comp = c->comp;
   return w;
 }
 
-// The unknowns of the wall rows of the state in buffer 0 (hlbm_init, hlbm_load).
-cudaError_t complete_walls(hlbm_ctx* c) {
-  WallArgs w = make_wall_args(c);
-  w.fin = c->pop[0];
-  w.mprev = c->mom[0];
-  w.comp_next = c->comp[0];
-  return launch_walls(w, c->storage, WALL_COMPLETE, false, c->stream);
-}
-
-// The streams of a wall-bounded context's edge launches and their events
-// (created once, outside capture).  High priority: the few blocks next to the
-// walls, the step's longest chain, must not queue behind those of the rows
-// between.
-cudaError_t ensure_wall_streams(hlbm_ctx* c) {
-  int lo = 0, hi = 0;
-  cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
-  for (int k = 0; k < 3 && e == cudaSuccess; ++k)
-    if (!c->wall_ev[k]) e = cudaEventCreateWithFlags(&c->wall_ev[k], cudaEventDisableTiming);
-  for (int k = 0; k < 2 && e == cudaSuccess; ++k)
-    if (!c->wall_stream[k]) e = cudaStreamCreateWithPriority(&c->wall_stream[k], cudaStreamNonBlocking, hi);
-  return e;
-}
-
-// One wall-bounded step (the moments of time t into mom[cur ^ 1]): the rows
-// next to the two walls on streams of their own, the rows between on the
-// context's.  None reads what another writes, and all read what the previous
-// step wrote, so the fork and the joins at the step's ends order everything;
-// under capture they become graph edges.
+// One wall-bounded step: the completion of the wall rows, the moments launch
+// (completed moments of time t into mom[cur ^ 1]), then the collide launch.
 cudaError_t wall_step(hlbm_ctx* c) {
   WallArgs w = make_wall_args(c);
   w.mcur = c->mom[c->cur ^ 1];
+  cudaError_t e = launch_walls(w, c->storage, WALL_COMPLETE, false, c->stream);
+  if (e == cudaSuccess) e = launch_walls(w, c->storage, WALL_MOMENTS, false, c->stream);
   w.fout = c->pop[c->cur ^ 1];
-  w.comp_next = c->comp[c->cur ^ 1];
-  const bool thermal = c->kind == KIND_THERMAL;
-  cudaError_t e = cudaEventRecord(c->wall_ev[2], c->stream);
-  for (int k = 0; k < 2; ++k) {
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->wall_stream[k], c->wall_ev[2], 0);
-    if (e == cudaSuccess) e = launch_walls(w, c->storage, k == 0 ? WALL_LOWER : WALL_UPPER, thermal, c->wall_stream[k]);
-  }
-  if (e == cudaSuccess) e = launch_walls(w, c->storage, WALL_BETWEEN, thermal, c->stream);
-  // join even after a failed launch, so that a capture in progress can end
-  for (int k = 0; k < 2; ++k) {
-    cudaError_t j = cudaEventRecord(c->wall_ev[k], c->wall_stream[k]);
-    if (j == cudaSuccess) j = cudaStreamWaitEvent(c->stream, c->wall_ev[k], 0);
-    if (e == cudaSuccess) e = j;
-  }
+  if (e == cudaSuccess) e = launch_walls(w, c->storage, WALL_COLLIDE, c->kind == KIND_THERMAL, c->stream);
   c->cur ^= 1;
   return e;
 }
@@ -757,7 +717,6 @@ hlbm_status hlbm_init(hlbm_ctx* c, const float* rho, const float* u, const float
     WallArgs w = make_wall_args(c);
     w.fout = c->pop[0];
     e = launch_wall_init(w, c->storage, a.rho, a.u, a.theta, c->mom[0], c->stream);
-    if (e == cudaSuccess) e = complete_walls(c);
   }
   if (e == cudaSuccess && !on_device) e = cudaStreamSynchronize(c->stream);  // host buffers are borrowed
   if (e != cudaSuccess) return cuda_fail(c, e, "init kernel");
@@ -802,7 +761,6 @@ hlbm_status hlbm_step(hlbm_ctx* c, int n) {
     HLBM_CUDA(c, cudaMemsetAsync(c->tile_ctr, 0, sizeof(unsigned long long), c->stream), "cudaMemsetAsync");
     c->ctr_reset = false;
   }
-  if (c->walls && n > 0) HLBM_CUDA(c, ensure_wall_streams(c), "wall streams");
   if (multistep_ok(c)) {
     while (n > 0) {
       NvtxRange chunk("hlbm_step: multi-step launch");
@@ -875,7 +833,8 @@ hlbm_status hlbm_moments(hlbm_ctx* c, float* rho, float* u, float* theta, int on
     w.rho_out = a.rho_out;
     w.u_out = a.u_out;
     w.theta_out = a.theta_out;
-    e = launch_walls(w, c->storage, WALL_MOMENTS, false, c->stream);
+    e = launch_walls(w, c->storage, WALL_COMPLETE, false, c->stream);
+    if (e == cudaSuccess) e = launch_walls(w, c->storage, WALL_MOMENTS, false, c->stream);
   } else if (c->aa) {
     e = aa_step(c, true, &a);
   } else {
@@ -905,6 +864,7 @@ hlbm_status hlbm_diag(hlbm_ctx* c, double* out) {
   if (c->walls) {
     WallArgs w = make_wall_args(c);
     w.partials = c->partials;
+    HLBM_CUDA(c, launch_walls(w, c->storage, WALL_COMPLETE, false, c->stream), "wall completion kernel");
     HLBM_CUDA(c, launch_walls(w, c->storage, WALL_MOMENTS, false, c->stream), "moments kernel");
   } else if (c->aa) {
     HLBM_CUDA(c, aa_step(c, true, &a), "moments kernel");
@@ -982,7 +942,6 @@ hlbm_status hlbm_load(hlbm_ctx* c, const void* host_buf, size_t bytes) {
   if (c->aa)
     HLBM_CUDA(c, cudaMemcpyAsync(c->aux[par ^ 1], static_cast<const char*>(host_buf) + 64 + pbytes, (size_t)4 * c->N,
                                  cudaMemcpyHostToDevice, c->stream), "cudaMemcpyAsync");
-  if (c->walls) HLBM_CUDA(c, complete_walls(c), "wall completion kernel");
   HLBM_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(int), c->stream), "cudaMemsetAsync");
   HLBM_CUDA(c, cudaMemsetAsync(c->tile_ctr, 0, sizeof(unsigned long long), c->stream), "cudaMemsetAsync");
   if (c->flags) HLBM_CUDA(c, cudaMemsetAsync(c->flags, 0, c->nflags * 4, c->stream), "cudaMemsetAsync");
@@ -1039,10 +998,6 @@ hlbm_status hlbm_destroy(hlbm_ctx* c) {
   if (!c) return HLBM_EINVAL;
   if (c->stream) cudaStreamSynchronize(c->stream);
   drop_graphs(c);
-  for (cudaStream_t ws : c->wall_stream)
-    if (ws) cudaStreamDestroy(ws);
-  for (cudaEvent_t ev : c->wall_ev)
-    if (ev) cudaEventDestroy(ev);
   if (c->own_arena && c->arena) cudaFree(c->arena);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;

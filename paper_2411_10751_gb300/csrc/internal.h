@@ -121,7 +121,7 @@ struct WallArgs {
   const void* fin;        // post-collision state of step t - 1, [Q][N]
   void* fout;             // collide: state written by this step
   const float* mprev;     // [4][N] rho, u_x, u_y, theta - 1 of the previous step (completed)
-  float* mcur;            // step: this step's [4][N] moments, written
+  float* mcur;            // moments: this step's [4][N] (may be null); collide: read for grad theta
   float* rho_out;         // moments readout (may be null)
   float* u_out;
   float* theta_out;
@@ -138,8 +138,7 @@ struct WallArgs {
   double wall_tb[2];      // their temperature minus 1
   float tb_ref;           // reference temperature of the stored deviations minus 1
   float e_ref;            // rho0 D c0^2 tb_ref: energy moment of the reference offset
-  const float* comp;      // completed unknowns of the six wall rows, [6][37][nx] (slot 3 side + r)
-  float* comp_next;       // those of the state written
+  float* comp;            // completed unknowns of the six wall rows, [6][37][nx] (slot 3 side + r)
 };
 
 // Arguments of the initialisation kernel.
@@ -196,12 +195,11 @@ cudaError_t launch_aa(const StepArgs& a, int kind, int storage, bool odd, bool m
 cudaError_t launch_aa_init(const StepArgs& a, int kind, int storage, const float* rho, const float* u,
                            const float* theta, cudaStream_t s);
 
-// Wall-bounded D2Q37 (walls.cu).  A step is LOWER, UPPER and BETWEEN, in any
-// order or at once (thermal: with H_i): they read a.fin and a.comp and write
-// a.fout, a.mcur and a.comp_next.  COMPLETE fills a.comp_next from a.fin and
-// a.mprev; MOMENTS is the readout (the readout pointers, partials) of a.fin and
-// a.comp.
-enum WallLaunch { WALL_LOWER, WALL_UPPER, WALL_BETWEEN, WALL_COMPLETE, WALL_MOMENTS };
+// Wall-bounded D2Q37 (walls.cu).  A step is, in this order, COMPLETE (the FP64
+// completion of the wall rows' unknowns into a.comp), MOMENTS (into a.mcur; also
+// the readout: the readout pointers, partials) and COLLIDE (thermal: with H_i).
+// MOMENTS and COLLIDE read a.comp.
+enum WallLaunch { WALL_COMPLETE, WALL_MOMENTS, WALL_COLLIDE };
 cudaError_t launch_walls(const WallArgs& a, int storage, WallLaunch what, bool thermal, cudaStream_t s);
 // Initial state of a wall-bounded context into a.fout and m [4][N] = rho,
 // u_x, u_y, theta - 1 of the initial fields.

@@ -32,14 +32,15 @@
 // (h* = (1 - omega) h + omega (g^eq - r) + beta S), and the completion is
 // the same in h as in g (r_i = r_ibar).
 //
-// Each step is three launches that run beside one another: the kEdge rows next
-// to the lower and to the upper wall (wall_edge_kernel, which also completes
-// the unknowns of the state that it writes, in FP64, for the next step) and the
-// rows between (wall_step_kernel).  Each pulls the populations once (the
-// unknowns from the completion buffer), forms the moments (rho, u, theta - 1)
-// of time t, grad theta (second-order central differences, one-sided into the
-// fluid at the wall rows) from them, collides (Eq. 4.4 with F_i and H_i) and
-// stores.
+// Each step is three launches: wall_complete_kernel completes the unknowns of
+// the six wall rows in FP64 into a small buffer; wall_moments_kernel pulls
+// every node's populations (the unknowns from that buffer) and writes its
+// moments (rho, u, theta - 1) of time t, which are the next step's targets and
+// the neighbour temperatures of grad theta; wall_collide_kernel pulls again,
+// collides (Eq. 4.4 with F_i and H_i) and stores.  grad theta is a
+// second-order central difference, one-sided into the fluid at the wall rows.
+// Two reads of the populations per step: these domains are the paper's
+// validation cases, a few thousand to a few hundred thousand nodes.
 #include "internal.h"
 #include "lattice.cuh"
 #include "step_common.cuh"
@@ -139,9 +140,8 @@ __device__ __forceinline__ void wall_accel(const WallArgs& a, int node, int y, f
 // warps on the four quarters run it four times as fast as one: the warps take
 // the x and the y moments of the target and of the previous state, then the
 // differences beside the scale's division, then one |c_x| each.  The longest
-// chain is 53 instructions.  A step of 200 x 102 takes 7.4 us with it, 11.1 us
-// with all 170 instructions in one warp, and took 49 us (47 us of them the
-// completion) with one thread per node and a whole expansion per population.
+// chain is 53 instructions; with one thread per node and a whole expansion per
+// population the launch took 47 us.
 constexpr int kCols = 4;    // columns of a block
 constexpr int kCompWarps = 4;
 
@@ -260,7 +260,7 @@ __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, in
   // phase 5: the velocities (+-cx, k), cx = wq: g_i = g*_ibar + rho_p (s P_i - P_ibar)
   const int x = x0 + col;
   if (lane < 6 * kCols && x < a.nx) {
-    float* out = a.comp_next + (size_t)(3 * side + r) * 37 * a.nx + x;
+    float* out = a.comp + (size_t)(3 * side + r) * 37 * a.nx + x;
     const int at = r * kCols + col;
     static_for<4>([&](auto Cx) {
       constexpr int cx = Cx;
@@ -282,9 +282,7 @@ __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, in
   }
 }
 
-// The completion from a stored state and its moments (after hlbm_init and
-// hlbm_load; a step completes the state that it writes itself): blockIdx.y the
-// wall.
+// The completion from a stored state and its moments: blockIdx.y the wall.
 template <int ST>
 __global__ void __launch_bounds__(32 * kCompWarps) wall_complete_kernel(const __grid_constant__ WallArgs a) {
   __shared__ CompIn in;
@@ -421,6 +419,12 @@ __global__ void __launch_bounds__(kBX * kBY, 4) wall_moments_kernel(const __grid
     const int node = y * a.nx + x;
     const WallMoments m = wall_moments(a, g, node, y);
     const size_t N = (size_t)a.N;
+    if (a.mcur) {
+      a.mcur[node] = m.rho;
+      a.mcur[N + node] = m.ux;
+      a.mcur[2 * N + node] = m.uy;
+      a.mcur[3 * N + node] = m.tb;
+    }
     if (a.rho_out) a.rho_out[node] = m.rho;
     if (a.u_out) {
       a.u_out[node] = m.ux;
@@ -453,13 +457,28 @@ __global__ void __launch_bounds__(kBX * kBY, 4) wall_moments_kernel(const __grid
   }
 }
 
-// grad theta's term and the collision of one node: g (the local deviations of
-// wall_moments) becomes the post-collision state
-template <bool THERMAL>
-__device__ __forceinline__ void wall_collide(const WallArgs& a, const WallMoments& m, float gtx, float gty, float (&g)[37]) {
+template <int ST, bool THERMAL>
+__global__ void __launch_bounds__(kBX * kBY, 3) wall_collide_kernel(const __grid_constant__ WallArgs a) {
+  const int x = blockIdx.x * kBX + threadIdx.x, y = blockIdx.y * kBY + threadIdx.y;
+  if (x >= a.nx || y >= a.ny) return;
+  const int nx = a.nx, ny = a.ny;
+  const size_t N = (size_t)a.N;
+  const int node = y * nx + x;
+  float g[37];
+  wall_gather<ST>(a, x, y, g);
+  const WallMoments m = wall_moments(a, g, node, y);
   NodeSrcT<float> s;
   s.hG[0] = s.hG[1] = s.hG[2] = 0.f;
   if constexpr (THERMAL) {
+    const float* tb = a.mcur + 3 * N;
+    const float gtx = 0.5f * (tb[y * nx + wrapx(x + 1, nx)] - tb[y * nx + wrapx(x - 1, nx)]);
+    float gty;
+    if (y == 0)
+      gty = 0.5f * (-3.f * tb[node] + 4.f * tb[node + nx] - tb[node + 2 * nx]);
+    else if (y == ny - 1)
+      gty = -0.5f * (-3.f * tb[node] + 4.f * tb[node - nx] - tb[node - 2 * nx]);
+    else
+      gty = 0.5f * (tb[node + nx] - tb[node - nx]);
     // s^(3) += rho theta (1 - 1/Pr) [delta grad_xi theta], grad_xi = c0 grad
     const float hc = m.rho * (1.f + m.tb) * (a.h_coef * (float)L::c0);
     s.hG[0] = hc * gtx;
@@ -481,177 +500,13 @@ __device__ __forceinline__ void wall_collide(const WallArgs& a, const WallMoment
   const float om1 = 1.f - a.omega;
   K[0] = fmaf(-om1, m.acc, K[0]);
   apply_poly_h<L, 15>(g, K, om1, m.dr);
-}
-
-__device__ __forceinline__ void store_moments(const WallArgs& a, const WallMoments& m, int node) {
-  const size_t N = (size_t)a.N;
-  a.mcur[node] = m.rho;
-  a.mcur[N + node] = m.ux;
-  a.mcur[2 * N + node] = m.uy;
-  a.mcur[3 * N + node] = m.tb;
-}
-
-// The step of the kEdge rows next to one wall, and the completion of the state
-// it writes.  A block owns kCols columns.  Its first warp takes the 16 nodes
-// and, with H_i, the ring of 12 around them for theta; given their moments,
-// its other four warps form the completion's brackets in FP64 while the first
-// collides, and complete the unknowns of rows 0 .. 2 from the new state.  So
-// no launch of a step waits for another one, and the FP64 work is spread over
-// nx / 2 blocks.
-constexpr int kEdge = 4;
-constexpr int kEdgeThreads = 32 * (1 + kCompWarps);
-
-// the block's barrier, from the different code of its warps
-__device__ __forceinline__ void edge_barrier() { asm volatile("barrier.sync 1, 160;" ::: "memory"); }
-
-template <int ST, bool THERMAL>
-__global__ void __launch_bounds__(kEdgeThreads) wall_edge_kernel(const __grid_constant__ WallArgs a, int side) {
-  constexpr int TW = kCols + 2;
-  __shared__ float tbs[(kEdge + 1) * TW];       // theta - 1 by rows from the wall, columns x0 - 1 .. x0 + kCols
-  __shared__ CompIn in;
-  __shared__ CompShared sh;
-  using T = typename Codec<ST>::T;
-  const int nx = a.nx, ny = a.ny;
-  const size_t N = (size_t)a.N;
-  const int lane = threadIdx.x & 31, x0 = blockIdx.x * kCols;
-  if (threadIdx.x < 32) {
-    // lanes 0 .. 15 the nodes, 16 .. 19 row kEdge, 20 .. 23 and 24 .. 27 the
-    // columns to the left and right
-    int r, c;
-    if (lane < kEdge * kCols) {
-      r = lane / kCols;
-      c = lane - r * kCols;
-    } else if (lane < kEdge * kCols + kCols) {
-      r = kEdge;
-      c = lane - kEdge * kCols;
-    } else {
-      const int q = lane - (kEdge + 1) * kCols;
-      r = q & (kEdge - 1);
-      c = q < kEdge ? -1 : kCols;
-    }
-    const int y = side == 0 ? r : ny - 1 - r;
-    int x = x0 + c;
-    // a domain of fewer than 2 kEdge rows: the lower wall's block stores the rows up to kEdge - 1
-    const bool store = lane < kEdge * kCols && x < nx && (side == 0 || y >= kEdge);
-    // column nx is column 0, the right neighbour of the last one
-    const bool needed = lane < (kEdge + 1) * kCols + 2 * kEdge && (store || (THERMAL && x <= nx));
-    if (x < 0) x += nx;
-    else if (x >= nx) x -= nx;
-    const int node = y * nx + x;
-    float g[37];
-    WallMoments m;
-    if (needed) {
-      wall_gather<ST>(a, x, y, g);
-      m = wall_moments(a, g, node, y);
-      if constexpr (THERMAL) tbs[r * TW + c + 1] = m.tb;
-      if (lane < 3 * kCols) {
-        in.mom[lane][0] = m.rho;
-        in.mom[lane][1] = m.ux;
-        in.mom[lane][2] = m.uy;
-        in.mom[lane][3] = m.tb;
-      }
-    }
-    edge_barrier();
-    if (store) {
-      float gtx = 0.f, gty = 0.f;
-      if constexpr (THERMAL) {
-        const float* tb = tbs + r * TW + c + 1;
-        gtx = 0.5f * (tb[1] - tb[-1]);
-        if (r == 0) {
-          gty = (side == 0 ? 0.5f : -0.5f) * (-3.f * tb[0] + 4.f * tb[TW] - tb[2 * TW]);
-        } else {
-          gty = side == 0 ? 0.5f * (tb[TW] - tb[-TW]) : 0.5f * (tb[-TW] - tb[TW]);
-        }
-      }
-      wall_collide<THERMAL>(a, m, gtx, gty, g);
-      store_moments(a, m, node);
-      const uint32_t salt = std::is_same<T, float>::value ? 0u : node_salt(node, g[0]);
-      if (HLBM_IN(node, a.N, DBG_STORE)) {
-        T* __restrict__ fout = static_cast<T*>(a.fout) + node;
-        static_for<37>([&](auto I) {
-          constexpr int i = I;
-          const T v = round_store<T>(g[i], pop_bits(salt, i));
-          fout[(size_t)i * N] = v;
-          if (lane < 3 * kCols) in.post[i][lane] = to_float(v);
-        });
-      }
-    }
-    edge_barrier();
-  } else {
-    complete_columns(a, side, x0, (threadIdx.x >> 5) - 1, lane, in, sh, [] { edge_barrier(); }, [] { edge_barrier(); });
-  }
-}
-
-// The step of the rows kEdge .. ny - 1 - kEdge, whose pulls and ring cross no
-// wall: moments, grad theta and collision in one pass.  A block owns kBX x kBY
-// nodes, one thread each, whose populations stay in registers; with H_i, three
-// more warps pull the 80 nodes of the 4-neighbour ring around them for theta
-// alone (their lines are the neighbour blocks', in L1 or L2), so the
-// populations are read from memory once per step (at 1024 x 1026 a moments and a
-// collide launch took 33 + 57 us; a whole step takes 72.7 us).
-template <bool THERMAL>
-constexpr int wall_threads() {
-  return kBX * kBY + (THERMAL ? 96 : 0);
-}
-
-template <int ST, bool THERMAL>
-__global__ void __launch_bounds__(wall_threads<THERMAL>(), THERMAL ? 2 : 3)
-    wall_step_kernel(const __grid_constant__ WallArgs a) {
-  constexpr int SW = kBX + 2, RING = 2 * kBX + 2 * kBY;
-  __shared__ float tbs[THERMAL ? (kBY + 2) * SW : 1];   // theta - 1 of the block and its ring
-  const int nx = a.nx, yhi = a.ny - kEdge;
-  const size_t N = (size_t)a.N;
-  const int tid = threadIdx.x;
-  const int x0 = blockIdx.x * kBX, y0 = kEdge + kBY * (int)blockIdx.y;
-  // region coordinates (0 .. kBX + 1, 0 .. kBY + 1) of this thread's node
-  int i, j;
-  if (tid < kBX * kBY) {
-    i = (tid & (kBX - 1)) + 1;
-    j = tid / kBX + 1;
-  } else {
-    const int q = tid - kBX * kBY;
-    if (q >= RING) i = j = -1;
-    else if (q < 2 * kBX) {
-      i = (q & (kBX - 1)) + 1;
-      j = q < kBX ? 0 : kBY + 1;
-    } else {
-      const int p = q - 2 * kBX;
-      i = p < kBY ? 0 : kBX + 1;
-      j = (p & (kBY - 1)) + 1;
-    }
-  }
-  const int y = y0 + j - 1;
-  int x = x0 + i - 1;
-  const bool store = tid < kBX * kBY && x < nx && y < yhi;
-  // column nx is column 0, the right neighbour of the last one; rows past yhi are not touched
-  const bool needed = j >= 0 && y <= yhi && (store || (THERMAL && x <= nx));
-  if (x < 0) x += nx;
-  else if (x >= nx) x -= nx;
-  const int node = y * nx + x;
-  float g[37];
-  WallMoments m;
-  if (needed) {
-    gather<L, Codec<ST>>(static_cast<const typename Codec<ST>::T*>(a.fin), a.N, nx, a.ny, 1, x, y, 0, g);
-    m = wall_moments(a, g, node, y);
-    if constexpr (THERMAL) tbs[j * SW + i] = m.tb;
-  }
-  if constexpr (THERMAL) __syncthreads();
-  if (!store) return;
-  store_moments(a, m, node);
-  float gtx = 0.f, gty = 0.f;
-  if constexpr (THERMAL) {
-    const float* tb = tbs + j * SW + i;
-    gtx = 0.5f * (tb[1] - tb[-1]);
-    gty = 0.5f * (tb[SW] - tb[-SW]);
-  }
-  wall_collide<THERMAL>(a, m, gtx, gty, g);
   using T = typename Codec<ST>::T;
   if (!HLBM_IN(node, a.N, DBG_STORE)) return;
   T* __restrict__ fout = static_cast<T*>(a.fout) + node;
   const uint32_t salt = std::is_same<T, float>::value ? 0u : node_salt(node, g[0]);
   static_for<37>([&](auto I) {
-    constexpr int q = I;
-    fout[(size_t)q * N] = round_store<T>(g[q], pop_bits(salt, q));
+    constexpr int i = I;
+    fout[(size_t)i * N] = round_store<T>(g[i], pop_bits(salt, i));
   });
 }
 
@@ -697,29 +552,14 @@ __global__ void __launch_bounds__(256) wall_init_kernel(const __grid_constant__ 
   });
 }
 
-template <int ST, bool THERMAL>
-cudaError_t launch_wall_step(const WallArgs& a, WallLaunch what, cudaStream_t s) {
-  if (what == WALL_BETWEEN) {
-    if (a.ny <= 2 * kEdge) return cudaSuccess;
-    const dim3 grid((a.nx + kBX - 1) / kBX, (a.ny - 2 * kEdge + kBY - 1) / kBY);
-    wall_step_kernel<ST, THERMAL><<<grid, wall_threads<THERMAL>(), 0, s>>>(a);
-  } else {
-    wall_edge_kernel<ST, THERMAL><<<(a.nx + kCols - 1) / kCols, kEdgeThreads, 0, s>>>(a, what == WALL_UPPER ? 1 : 0);
-  }
-  return cudaGetLastError();
-}
-
 template <int ST>
 cudaError_t launch_walls_st(const WallArgs& a, WallLaunch what, bool thermal, cudaStream_t s) {
-  if (what == WALL_COMPLETE) {
-    wall_complete_kernel<ST><<<dim3((a.nx + kCols - 1) / kCols, 2), 32 * kCompWarps, 0, s>>>(a);
-    return cudaGetLastError();
-  }
-  if (what == WALL_MOMENTS) {
-    wall_moments_kernel<ST><<<dim3((a.nx + kBX - 1) / kBX, (a.ny + kBY - 1) / kBY), dim3(kBX, kBY), 0, s>>>(a);
-    return cudaGetLastError();
-  }
-  return thermal ? launch_wall_step<ST, true>(a, what, s) : launch_wall_step<ST, false>(a, what, s);
+  const dim3 block(kBX, kBY), grid((a.nx + kBX - 1) / kBX, (a.ny + kBY - 1) / kBY);
+  if (what == WALL_COMPLETE) wall_complete_kernel<ST><<<dim3((a.nx + kCols - 1) / kCols, 2), 32 * kCompWarps, 0, s>>>(a);
+  else if (what == WALL_MOMENTS) wall_moments_kernel<ST><<<grid, block, 0, s>>>(a);
+  else if (thermal) wall_collide_kernel<ST, true><<<grid, block, 0, s>>>(a);
+  else wall_collide_kernel<ST, false><<<grid, block, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace

@@ -1,7 +1,7 @@
 """Wall-bounded step at the edges of its launches: domains of the fewest rows and
 columns, block rows and columns that are cut short, both wall kinds, with and
-without the thermal source; and the completion of the wall rows inside a step
-against that from a stored state.
+without the thermal source; and a split run (the wall rows completed from a saved
+state) against the whole one.
 
 Against the FP64 oracle the bar is the parity tests' 1e-5 per field (FP32
 storage, velocity on the scale max(|u|, 0.01)); a split run must equal the
@@ -15,7 +15,7 @@ from oracle.solver import Oracle
 
 pytestmark = pytest.mark.gpu
 
-# rows: 4 next to each wall, 8 per block between them; columns: 4 per edge block, 32 per block
+# 8 rows and 32 columns per block, 4 columns per block of the completion
 SIZES = [(7, 7), (8, 8), (9, 9), (33, 11), (31, 16), (66, 17), (65, 25)]
 
 
@@ -71,7 +71,7 @@ def test_completion_in_the_step_equals_that_from_a_saved_state(HLBM, nx, ny, sto
     g.init(c.rho, c.u, c.theta)
     g.step(33)
     part = g.save()
-    g.step(3)          # other contents in both completion buffers
+    g.step(3)          # other contents in the completion buffer
     g.load(part)
     g.step(7)
     assert g.save() == whole

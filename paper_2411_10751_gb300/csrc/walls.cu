@@ -157,11 +157,9 @@ struct CompShared {
 
 __device__ __forceinline__ void comp_barrier() { asm volatile("barrier.sync 2, 128;" ::: "memory"); }
 
-// Called by four whole warps (wq = 0 .. 3); moments_ready() and state_ready()
-// return once in.mom and in.post are written.  x0: first column of the block.
-template <class M, class P>
+// Called by four whole warps (wq = 0 .. 3).  x0: first column of the block.
 __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, int x0, int wq, int lane, const CompIn& in,
-                                                 CompShared& sh, M&& moments_ready, P&& state_ready) {
+                                                 CompShared& sh) {
   const int lc = lane / 6, t = lane - 6 * lc;
   const int col = lc < kCols ? lc : kCols - 1;          // lanes past the last column repeat it
   const int r = t < 3 ? 0 : (t < 5 ? 1 : 2);            // rows from the wall node
@@ -175,7 +173,6 @@ __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, in
   const double w0 = pick3(k, kRowSum<1, 0>, kRowSum<2, 0>, kRowSum<3, 0>);
   const double w2 = pick3(k, kRowSum<1, 2>, kRowSum<2, 2>, kRowSum<3, 2>);
   const double w4 = pick3(k, kRowSum<1, 4>, kRowSum<2, 4>, kRowSum<3, 4>);
-  moments_ready();
   // phase 1: the Gaussian moments of one component of one state.  P(c; u) is
   // even in (c, u) per axis, so the rows are evaluated at c_y = +k, with u_y
   // mirrored at the upper wall, and the previous state, taken at the opposite
@@ -256,7 +253,6 @@ __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, in
   }
   comp_barrier();
   const double rp = p[0];
-  state_ready();
   // phase 5: the velocities (+-cx, k), cx = wq: g_i = g*_ibar + rho_p (s P_i - P_ibar)
   const int x = x0 + col;
   if (lane < 6 * kCols && x < a.nx) {
@@ -296,7 +292,7 @@ __global__ void __launch_bounds__(32 * kCompWarps) wall_complete_kernel(const __
     else in.mom[at][i - 37] = __ldg(a.mprev + (size_t)(i - 37) * N + y * a.nx + x);
   }
   __syncthreads();
-  complete_columns(a, side, x0, threadIdx.x >> 5, threadIdx.x & 31, in, sh, [] {}, [] {});
+  complete_columns(a, side, x0, threadIdx.x >> 5, threadIdx.x & 31, in, sh);
 }
 
 // The 37 populations of node (x, y) at time t after streaming, the unknowns

@@ -187,10 +187,27 @@ __device__ __forceinline__ bool tile_boxed(const StepArgs& a, int x0, int y0) {
          (y0 - H + 3 + Cf::HB <= a.ny);
 }
 
+// Whether a staged kernel's edge tiles gather with 64-bit address sums.  The
+// register limits of these kernels are those of the staged tiles' collision, and
+// beside it the uniform plane addresses of the 32-bit form spill or lengthen the
+// gather in some of them (us per step, 32-bit / 64-bit: FP32 body force, 8 rows
+// and two nodes, 512 x 512 11.8 / 11.3, 544 x 544 13.7 / 12.7; one node on 8 rows,
+// thermal 64 x 64 FP16 and pseudopotential 64 x 64 FP16 1.31 and 1.40 times the
+// 64-bit form's time, 1024 x 1024 1.03 and 1.07 times; two nodes on 16 rows, body
+// force 513 x 511 FP16 1.05 times).  The others gain 1 to 5% by it (8 rows, two
+// nodes: body force FP16 384 x 384 7.4 -> 7.1, pseudopotential FP16 640 x 640
+// 31.2 -> 30.2; 16 rows, one node, thermal 0.94 to 0.98 times).
+template <int ST, int KIND, int BY, int NPT>
+constexpr bool edge_sum64() {
+  if (BY == 8 && NPT == 2) return ST == ST_F32 && KIND == KIND_LOCAL;
+  if (BY == 8) return KIND != KIND_LOCAL;
+  return BY == 16 && NPT == 2 && KIND != KIND_SC;
+}
+
 // Edge tile: every region node gathers its Q pulled populations of `fin_v`
 // with periodic wrap (independent loads through codec C) and writes them into
 // the staged layout.
-template <class Cf, int NT, class C = typename Cf::C>
+template <class Cf, int NT, bool SUM64, class C = typename Cf::C>
 __device__ __forceinline__ void fill_tile_wrapped(const StepArgs& a, const void* fin_v, typename Cf::T* sp, int x0,
                                                   int y0, int tid) {
   using L = D2Q37;
@@ -201,7 +218,7 @@ __device__ __forceinline__ void fill_tile_wrapped(const StepArgs& a, const void*
     const int ry = k / Cf::RW, rx = k - ry * Cf::RW;
     const int X = wrapm(x0 - H + rx, a.nx), Y = wrapm(y0 - H + ry, a.ny);
     float gk[37];
-    gather<L, C>(fin, a.N, a.nx, a.ny, 1, X, Y, 0, gk);
+    gather<L, C, SUM64>(fin, a.N, a.nx, a.ny, 1, X, Y, 0, gk);
     const int base = ry * Cf::WB + rx;
     static_for<37>([&](auto I) {
       constexpr int i = I;
@@ -483,7 +500,7 @@ __global__ void __launch_bounds__(32 * BY / NPT, (min_ctas2<ST, KIND, MOM, BY, N
       return;
     }
   } else {
-    fill_tile_wrapped<Cf, NT>(a, a.fin, sp, x0, y0, tid);
+    fill_tile_wrapped<Cf, NT, !MOM && edge_sum64<ST, KIND, BY, NPT>()>(a, a.fin, sp, x0, y0, tid);
     __syncthreads();
   }
   process_tile<ST, KIND, MOM, BY, NPT, true>(a, &tmap_out, smem, x0, y0, a.fout, [] {});
@@ -655,7 +672,7 @@ __global__ void __launch_bounds__(32 * BY / NPT, (min_ctas_persistent<ST, KIND, 
       }
       phase ^= 1u;
     } else {
-      fill_tile_wrapped<Cf, NT>(a, a.fin, sp, x0, y0, tid);
+      fill_tile_wrapped<Cf, NT, edge_sum64<ST, KIND, BY, NPT>()>(a, a.fin, sp, x0, y0, tid);
       __syncthreads();
     }
     constexpr bool SEP = persistent_sep_out<ST>();
@@ -815,7 +832,7 @@ __global__ void __launch_bounds__(32 * BY / NPT, (min_ctas2<ST, KIND, false, BY,
       }
       phase ^= 1u;
     } else {
-      fill_tile_wrapped<Cf, NT, CodecCG<ST>>(a, (s & 1) ? a.fout : a.fin, sp, x0, y0, tid);
+      fill_tile_wrapped<Cf, NT, edge_sum64<ST, KIND, BY, NPT>(), CodecCG<ST>>(a, (s & 1) ? a.fout : a.fin, sp, x0, y0, tid);
       __syncthreads();
     }
     process_tile<ST, KIND, false, BY, NPT, false>(a, nullptr, smem, x0, y0, (s & 1) ? const_cast<void*>(a.fin) : a.fout,

@@ -267,7 +267,10 @@ __device__ __forceinline__ int wrap_up(int v, int n) {
 
 // ------------------------------------------------------------------ gather
 // g_i(x) = stored_i(x - c_i), periodic.  x in [0,nx), y in [0,ny), z in [0,nz).
-template <class L, class C>
+// A plane's address is uniform and the node's offset an unsigned 32-bit index;
+// SUM64: one 64-bit sum per population, for kernels whose registers the uniform
+// form overdraws (edge_sum64, step2d.cuh).
+template <class L, class C, bool SUM64 = false>
 __device__ __forceinline__ void gather(const typename C::T* __restrict__ f, long long N, int nx, int ny,
                                        int nz, int x, int y, int z, float (&g)[L::Q]) {
   int xs[7], ys[7], zs[7];
@@ -282,7 +285,10 @@ __device__ __forceinline__ void gather(const typename C::T* __restrict__ f, long
     constexpr int cx = L::c(i, 0), cy = L::c(i, 1), cz = L::c(i, 2);
     int off = ys[cy + 3] + xs[cx + 3];
     if constexpr (L::D == 3) off += zs[cz + 3];
-    g[i] = C::ld(f + (size_t)i * (size_t)N + (unsigned)HLBM_IDX(off, N, DBG_GATHER));
+    if constexpr (SUM64)
+      g[i] = C::ld(f + HLBM_IDX((size_t)i * (size_t)N + off, (long long)L::Q * N, DBG_GATHER));
+    else
+      g[i] = C::ld(f + (size_t)i * (size_t)N + (unsigned)HLBM_IDX(off, N, DBG_GATHER));
   });
 }
 

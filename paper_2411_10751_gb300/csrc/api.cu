@@ -265,6 +265,30 @@ void drop_graphs(hlbm_ctx* c) {
     }
 }
 
+// Tiles of pitch `pitch` along an axis of n nodes whose box [t pitch - lo, t pitch + width) lies inside it.
+long long boxed_tiles(int n, int pitch, int lo, int width) {
+  const long long first = (lo + pitch - 1) / pitch, last = n >= width ? (n - width) / pitch : -1;
+  return std::max(0LL, last - first + 1);
+}
+
+// Share of a D2Q37 domain's 32 x 8 tiles that a persistent kernel can stage ahead
+// by TMA (tile_boxed, step2d.cuh); it fills the others synchronously, on the
+// periodic edge.  kind: the one that the boxes are cut for.
+double boxed_share(const hlbm_ctx* c, int kind) {
+  int wb = 0, hb = 0, ob = 0;
+  step_box_d2q37(kind, c->storage, false, 8, &wb, &hb, &ob);
+  const int H = (hb - 8) / 2, A = 16 / (int)c->elem;
+  const double tiles = (double)((c->nx + 31) / 32) * ((c->ny + 7) / 8);
+  return (double)boxed_tiles(c->nx, 32, H + 3 + A - 1, 3 - H + wb) * boxed_tiles(c->ny, 8, H + 3, 3 - H + hb) / tiles;
+}
+
+// The persistent kernels' gain is the next tile in flight, so they need most
+// tiles boxed.  us per step, one CTA per tile against persistent, by the boxed
+// share, thermal and pseudopotential, FP32: 0: 80 x 6000 39.7 / 44.5, 64.6 / 69.9;
+// 1/2: 120 x 4500 39.7 / 42.9, 62.6 / 66.4; 3/5: 140 x 4000 43.9 / 47.6, 66.7 / 67.4;
+// 2/3: 176 x 3000 37.8 / 37.0, 58.9 / 58.1; 7/9: 264 x 1500 29.1 / 26.7, 46.1 / 44.8.
+constexpr double kMinBoxed = 0.62;
+
 // Whether a context without a schedule runs the persistent kernels (D2Q37
 // staged tiles, D3Q39 whole rows).  Their CTAs take ordered tiles and hold the
 // next one in flight, which pays once a step streams from HBM, i.e. when the two
@@ -279,7 +303,8 @@ void drop_graphs(hlbm_ctx* c) {
 // others (1536 x 1536 109.1 / 112.4).
 int auto_persistent(const hlbm_ctx* c) {
   if (2.0 * c->Q * (double)c->N * (double)c->elem < 96e6) return 0;
-  return c->lattice == HLBM_D3Q39 || (c->storage == ST_F32 && c->kind != KIND_LOCAL) ? 1 : 0;
+  if (c->lattice == HLBM_D3Q39) return 1;
+  return c->storage == ST_F32 && c->kind != KIND_LOCAL && boxed_share(c, c->kind) >= kMinBoxed ? 1 : 0;
 }
 
 StepArgs make_args(const hlbm_ctx* c) {

@@ -499,12 +499,22 @@ cudaError_t wall_step(hlbm_ctx* c) {
 
 // Whether the in-place step runs its persistent TMA-staged form: FP32, from the
 // size on where its one buffer streams from HBM (us per step, pulls / staged:
-// body force 1024 x 1024 55.6 / 50.8, thermal 63.4 / 56.8, pseudopotential 73.1 /
-// 64.5; 2048 x 2048 208.9 / 199.1, 240.2 / 214.3, 272.4 / 239.4; inside L2, 512 x 512,
-// 10.8 / 15.6, 12.9 / 17.9, 15.8 / 20.4).  In 16 bits the pulls are as fast or
-// faster (1024 x 1024 37.0 / 46.3, 47.9 / 52.9, 59.8 / 64.2).
+// body force 1024 x 640 (97 MB) 29.4 / 31.9, 20000 x 36 (107 MB) 35.7 / 38.4, 128 x
+// 6144 (116 MB) 39.0 / 38.5, 1024 x 1024 54.5 / 49.7; thermal 1024 x 640 36.7 / 36.0,
+// 1024 x 1024 63.0 / 56.4; pseudopotential 42.9 / 41.8, 69.4 / 64.3; inside L2, 512 x
+// 512, 10.8 / 15.6, 12.9 / 17.9, 15.8 / 20.4).  Its CTAs run a tile that cannot be
+// boxed much as the pulls do, but for the columns past the domain's edge, whose
+// loads it pays for: few boxed tiles are a loss where the last tile column is cut
+// short (body force, thermal, pseudopotential: none boxed, 36 x 20000 42.7 / 52.4,
+// 56.8 / 61.1, 67.7 / 72.1; 3/5, 140 x 5800 43.6 / 45.9, 49.4 / 51.5, 56.1 / 58.4; 5/7,
+// 200 x 4000 43.7 / 43.4, 49.8 / 48.7, 56.3 / 55.3) and none where it is whole (none
+// boxed, 32 x 24000 39.2 / 34.9, 45.4 / 41.3, 51.2 / 48.4; 1/3, 96 x 8000 38.3 / 37.7,
+// 44.8 / 42.7, 50.4 / 48.8).  In 16 bits the pulls are as fast or faster (1024 x
+// 1024 37.0 / 46.3, 47.9 / 52.9, 59.8 / 64.2).
 bool aa_staged(const hlbm_ctx* c) {
-  return c->tma_ok && !c->debug_skip_tma && c->storage == ST_F32 && (double)c->Q * (double)c->N * 4.0 >= 96e6;
+  if (!c->tma_ok || c->debug_skip_tma || c->storage != ST_F32) return false;
+  if ((double)c->Q * (double)c->N * 4.0 < (c->kind == KIND_LOCAL ? 108e6 : 96e6)) return false;
+  return c->nx % 32 == 0 || boxed_share(c, KIND_LOCAL) >= kMinBoxed;   // the boxes of a tile's own slots
 }
 
 // One in-place step of parity cur: reads aux[cur ^ 1], writes aux[cur].

@@ -1,6 +1,6 @@
 """The schedule that a context without one gets must not lose to the one-CTA-per-tile
-schedule (8 rows, two nodes per thread) on domains where the persistent kernels
-cannot stage most of their tiles.
+schedule (8 rows, two nodes per thread), nor the in-place step to its pulled form,
+on domains where the persistent kernels cannot stage most of their tiles.
 
 The bar is 8%: repeated timings of one schedule differ by less than 1%, and the
 losses that these domains had were 11% and more.
@@ -57,3 +57,13 @@ def test_narrow_domain_default_keeps_up_with_one_cta_per_tile(HLBM, kind, nx, ny
         c = W.droplet(nx=nx, ny=ny, r0=0.25 * min(nx, ny), Tr=0.9)
     auto, grid = _us_per_step(HLBM, c), _us_per_step(HLBM, c, (8, 2, 1))
     assert auto < BAR * grid, (auto, grid)
+
+
+@pytest.mark.parametrize("nx,ny", [(36, 20000), (68, 12000)])
+def test_narrow_in_place_step_keeps_up_with_its_pulled_form(HLBM, monkeypatch, nx, ny):
+    c = W.kolmogorov(nx=nx, ny=ny, g0=1e-5)
+    c.params = dict(c.params, lag=True)
+    auto = _us_per_step(HLBM, c)
+    monkeypatch.setenv("HLBM_NO_TMA", "1")
+    pulled = _us_per_step(HLBM, c)
+    assert auto < BAR * pulled, (auto, pulled)

@@ -289,6 +289,26 @@ double boxed_share(const hlbm_ctx* c, int kind) {
 // 2/3: 176 x 3000 37.8 / 37.0, 58.9 / 58.1; 7/9: 264 x 1500 29.1 / 26.7, 46.1 / 44.8.
 constexpr double kMinBoxed = 0.62;
 
+// Whether a D3Q39 context without a schedule runs the whole-row kernel.  Planes
+// whose rows cross the y-edge are copied row by row, which costs most where a tile
+// has many rows (8 at nx = 32, 4 at nx = 64) of a small ny; what it saves most on is
+// a force field, which it stages beside them.  us per step, gather kernel / whole
+// rows.  nx = 32, FP32, field: 32 x 7 x 1600 21.8 / 43.0, 32 x 24 x 900 41.9 / 39.3,
+// 32 x 101 x 99 (100 MB) 17.0 / 21.7, 32 x 64 x 180 (115 MB) 20.9 / 20.3, 32 x 160 x
+// 160 49.1 / 40.7; no field: 32 x 300 x 60 31.2 / 31.9, 32 x 160 x 160 41.5 / 40.0.
+// nx = 64, FP32, field: 64^3 (82 MB) 12.4 / 14.1, 64 x 64 x 80 (102 MB) 17.8 / 16.7; no
+// field: 64 x 64 x 80 14.9 / 16.6, 64 x 64 x 100 (128 MB) 21.4 / 19.7, 64 x 9 x 1200
+// 46.1 / 47.7, 64 x 16 x 700 37.1 / 35.5.  nx >= 128, FP32, no field: 128 x 50 x 50 (100
+// MB) 15.8 / 15.3, 128 x 7 x 600 30.4 / 28.1, 128^3 100.6 / 94.7 (field 120.0 / 98.8).  FP16, field:
+// 64 x 64 x 160 (102 MB) 31.0 / 29.2; no field: 28.5 / 29.4, 64 x 128 x 128 (164 MB) 44.4 /
+// 43.1.
+bool auto_rows3(const hlbm_ctx* c, double bytes) {
+  const bool field = c->force_mode == FORCE_FIELD, tall = c->ny >= 3 * (256 / c->nx);
+  if (c->nx == 32) return field && tall && bytes >= 112e6;
+  if (field || (c->storage == ST_F32 && c->nx >= 128)) return bytes >= 96e6;
+  return tall && bytes >= 120e6;
+}
+
 // Whether a context without a schedule runs the persistent kernels (D2Q37
 // staged tiles, D3Q39 whole rows).  Their CTAs take ordered tiles and hold the
 // next one in flight, which pays once a step streams from HBM, i.e. when the two
@@ -296,14 +316,14 @@ constexpr double kMinBoxed = 0.62;
 // block scheduling is faster.  us per step, one CTA per tile against
 // persistent, FP32 unless stated: thermal 512 x 512 (78 MB) 16.7 / 18.0, 576 x 576
 // (98 MB) 21.4 / 19.6, 1024 x 1024 60.9 / 54.9; pseudopotential 576 x 576 35.9 /
-// 34.8, 1024 x 1024 95.5 / 89.4; D3Q39 64^3 (82 MB) 12.3 / 15.0, 128^3 136.2 / 98.8,
-// 128^3 FP16 97.1 / 79.9.  Not for D2Q37 in 16 bits, whose persistent form has 3
+// 34.8, 1024 x 1024 95.5 / 89.4 (D3Q39 above).  Not for D2Q37 in 16 bits, whose persistent form has 3
 // CTAs per SM instead of 4 (thermal 1024 x 1024 45.4 / 48.8), nor for the body
 // force alone, which gains at some sizes (1024 x 1024 54.1 / 53.1) and loses at
 // others (1536 x 1536 109.1 / 112.4).
 int auto_persistent(const hlbm_ctx* c) {
-  if (2.0 * c->Q * (double)c->N * (double)c->elem < 96e6) return 0;
-  if (c->lattice == HLBM_D3Q39) return 1;
+  const double bytes = 2.0 * c->Q * (double)c->N * (double)c->elem;
+  if (bytes < 96e6) return 0;
+  if (c->lattice == HLBM_D3Q39) return auto_rows3(c, bytes) ? 1 : 0;
   return c->storage == ST_F32 && c->kind != KIND_LOCAL && boxed_share(c, c->kind) >= kMinBoxed ? 1 : 0;
 }
 

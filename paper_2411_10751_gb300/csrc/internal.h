@@ -43,7 +43,9 @@ int per_device_cached(std::atomic<int> (&cache)[kMaxDevicesCached], F&& compute)
 // still runs (programmatic dependent launch, also inside a captured graph):
 // its blocks take free slots and run up to grid_dependency_wait()
 // (step_common.cuh) meanwhile.  The kernel must execute that wait before its
-// first access to memory that an earlier launch reads or writes.
+// first access to memory that an earlier launch reads or writes.  A refused
+// launch is this call's result only: the thread's last error is taken back, or the
+// next launch of another context would report it.
 template <class... P>
 cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const P&... args) {
   cudaLaunchConfig_t cfg{};
@@ -56,7 +58,9 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 enum Kind : int {

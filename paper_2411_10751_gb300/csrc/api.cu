@@ -616,6 +616,16 @@ cudaError_t launch_multistep(hlbm_ctx* c, int S) {
   return cudaSuccess;
 }
 
+// Restarts the persistent step's tile counter after a change of schedule: its
+// period is the tiles and CTAs of one launch, and a counter left by launches of
+// another period would start this one part of the way through its tiles.
+hlbm_status restart_counters(hlbm_ctx* c) {
+  if (!c->ctr_reset) return HLBM_OK;
+  HLBM_CUDA(c, cudaMemsetAsync(c->tile_ctr, 0, sizeof(unsigned long long), c->stream), "cudaMemsetAsync");
+  c->ctr_reset = false;
+  return HLBM_OK;
+}
+
 hlbm_status usable(hlbm_ctx* c) {
   if (!c) return HLBM_EINVAL;
   if (c->failed) return HLBM_ESTATE;
@@ -811,11 +821,7 @@ hlbm_status hlbm_step(hlbm_ctx* c, int n) {
   if (st != HLBM_OK) return st;
   if (n < 0) return fail(c, HLBM_EINVAL, "n must be >= 0");
   if (!c->initialised) return fail(c, HLBM_ESTATE, "hlbm_init has not been called");
-  if (c->ctr_reset) {
-    // the persistent launch's CTA count may have changed: restart the counter
-    HLBM_CUDA(c, cudaMemsetAsync(c->tile_ctr, 0, sizeof(unsigned long long), c->stream), "cudaMemsetAsync");
-    c->ctr_reset = false;
-  }
+  if ((st = restart_counters(c)) != HLBM_OK) return st;
   if (multistep_ok(c)) {
     while (n > 0) {
       NvtxRange chunk("hlbm_step: multi-step launch");
@@ -1097,6 +1103,7 @@ hlbm_status hlbm_adjoint_run(hlbm_ctx* c, int steps, int ckpt_every, void* works
   const int K = std::min(ckpt_every, steps);
   const AdjLayout L = adj_layout(c, steps, K);
   if (bytes < L.total) return fail(c, HLBM_ENOMEM, "adjoint workspace smaller than hlbm_adjoint_workspace_bytes()");
+  if ((st = restart_counters(c)) != HLBM_OK) return st;
   // a map depends only on (address, box, type, extent), so maps of an earlier
   // run's workspace stay valid for a workspace at the same address; the cache
   // is only trimmed back to the context's own buffers when it grows large

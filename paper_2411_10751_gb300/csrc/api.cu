@@ -616,12 +616,18 @@ cudaError_t launch_multistep(hlbm_ctx* c, int S) {
   return cudaSuccess;
 }
 
-// Restarts the persistent step's tile counter after a change of schedule: its
+// Restarts the device counters after a change of schedule.  The persistent step's
 // period is the tiles and CTAs of one launch, and a counter left by launches of
-// another period would start this one part of the way through its tiles.
+// another period would start this one part of the way through its tiles.  The
+// multi-step kernel's completion counters belong to tile rows: rows that the
+// schedule before did not have would be waited for from zero.
 hlbm_status restart_counters(hlbm_ctx* c) {
   if (!c->ctr_reset) return HLBM_OK;
   HLBM_CUDA(c, cudaMemsetAsync(c->tile_ctr, 0, sizeof(unsigned long long), c->stream), "cudaMemsetAsync");
+  if (c->multistep && c->flags) {
+    HLBM_CUDA(c, cudaMemsetAsync(c->flags, 0, c->nflags * 4, c->stream), "cudaMemsetAsync");
+    c->gen = 0;
+  }
   c->ctr_reset = false;
   return HLBM_OK;
 }

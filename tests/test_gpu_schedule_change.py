@@ -44,3 +44,22 @@ def test_adjoint_after_a_change_of_schedule(HLBM, K):
     assert g.save() == ref.save()
     ref.close()
     g.close()
+
+
+@pytest.mark.parametrize("first,then", [((16, 2, 3), (8, 2, 3)), ((8, 2, 3), (4, 1, 3)), ((8, 1, 3), (16, 1, 3))])
+def test_multi_step_kernel_after_a_change_of_rows(HLBM, first, then):
+    """Against the same steps on the same tiles by the kernel of one launch per step
+    (other tiles round theta on their frames differently)."""
+    c = W.thermal_decay(nx=128, ny=96)
+    ref = _context(HLBM, c, first[:2] + (2,))
+    ref.step(7)
+    ref.set_tile(*then[:2], 2)
+    ref.step(10)
+    g = _context(HLBM, c, first)
+    g.step(7)
+    g.set_tile(*then)
+    g.step(10)
+    g.synchronize()
+    assert g.save() == ref.save()
+    ref.close()
+    g.close()

@@ -132,7 +132,8 @@ def _multistep(case, sched) -> bool:
 
 def _launches(case, sched, steps) -> int:
     """Step-kernel launches of hlbm_step(steps): one per step, or one per
-    block of up to 1024 steps for the multi-step kernel."""
+    block of up to 1024 steps for the multi-step kernel.  (Without a schedule a
+    pseudopotential step may be two launches: at least one per step is claimed.)"""
     if case.params.get("walls"):
         return 3 * steps   # wall completion, moments, collision
     if not _multistep(case, sched):
@@ -749,6 +750,7 @@ def main():
                          "kernel": "wall_complete_kernel + wall_moments_kernel + wall_collide_kernel (three launches per step, the "
                                    "populations read in both)" if case.params.get("walls") else
                                    "aa_step_kernel (in place, one launch per step)" if case.params.get("lag") else
+                                   "the library's choice by size, kind and alignment" if not any(sched) else
                                    (("step3d_rows_kernel" if sched[2] >= 2 and case.nx in (32, 64, 128, 256)
                                      else "step3d_kernel") if case.lattice == "D3Q39" else
                                     ("step2d_multistep_kernel" if _multistep(case, sched) else

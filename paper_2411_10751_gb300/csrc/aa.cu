@@ -331,6 +331,7 @@ __global__ void __launch_bounds__(kBX * kBY / 2, 4)
     if (!tile_boxed<Cf>(a, x0, y0)) return;
     fence_proxy_async_smem();
     if (warp == 0) mbar_arrive_expect_tx(bar, Cf::TX_BYTES);
+    if (a.debug_skip_tma) return;   // test hook: the wait must expire
     static_for<37>([&](auto I) {
       constexpr int i = I;
       if (i % W != warp) return;

@@ -532,7 +532,7 @@ cudaError_t wall_step(hlbm_ctx* c) {
 // 44.8 / 42.7, 50.4 / 48.8).  In 16 bits the pulls are as fast or faster (1024 x
 // 1024 37.0 / 46.3, 47.9 / 52.9, 59.8 / 64.2).
 bool aa_staged(const hlbm_ctx* c) {
-  if (!c->tma_ok || c->debug_skip_tma || c->storage != ST_F32) return false;
+  if (!c->tma_ok || c->storage != ST_F32) return false;
   if ((double)c->Q * (double)c->N * 4.0 < (c->kind == KIND_LOCAL ? 108e6 : 96e6)) return false;
   return c->nx % 32 == 0 || boxed_share(c, KIND_LOCAL) >= kMinBoxed;   // the boxes of a tile's own slots
 }

@@ -135,7 +135,9 @@ hlbm_status hlbm_create(int lattice, int nx, int ny, int nz, double tau_hat,
 
 /* Uses caller-owned device memory of at least hlbm_workspace_bytes() bytes,
  * 256-byte aligned, instead of allocating.  The caller keeps it alive until
- * hlbm_destroy.  Must precede hlbm_init. */
+ * hlbm_destroy.  Must precede hlbm_init.  The psi field (the last 4 nx ny bytes,
+ * rounded up to 256, with HLBM_SRC_SC without HLBM_AA) may be left out: such a
+ * context never steps in two launches. */
 hlbm_status hlbm_bind_memory(hlbm_ctx* ctx, void* dev_ptr, size_t bytes);
 
 /* Orders all work of the context on this cudaStream_t (0: a private stream

@@ -98,7 +98,7 @@ namespace {
 
 struct Layout {
   size_t pop_bytes, off_pop1, off_g, off_part, off_red, off_flags, nflags, off_mom, mom_bytes, off_aux, aux_bytes,
-      off_comp, comp_bytes, total;
+      off_comp, comp_bytes, total, required;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -129,6 +129,9 @@ Layout layout(int lattice, int nx, int ny, int nz, const hlbm_source_params* p) 
   L.off_comp = L.off_aux + ((p->flags & HLBM_AA) ? 2 : 1) * L.aux_bytes;
   L.comp_bytes = (p->flags & HLBM_WALLS) ? align256((size_t)6 * 37 * (size_t)nx * 4) : 0;
   L.total = L.off_comp + L.comp_bytes;
+  // psi, the last of its layout, serves the step in two launches only: an arena
+  // without room for it runs the step in one
+  L.required = (p->flags & HLBM_SRC_SC) && !(p->flags & HLBM_AA) ? L.off_aux : L.total;
   return L;
 }
 
@@ -245,8 +248,8 @@ void carve(hlbm_ctx* c) {
   c->nflags = L.nflags;
   c->mom[0] = L.mom_bytes ? reinterpret_cast<float*>(c->arena + L.off_mom) : nullptr;
   c->mom[1] = L.mom_bytes ? reinterpret_cast<float*>(c->arena + L.off_mom + L.mom_bytes) : nullptr;
-  c->aux[0] = L.aux_bytes ? reinterpret_cast<float*>(c->arena + L.off_aux) : nullptr;
-  c->aux[1] = L.aux_bytes ? reinterpret_cast<float*>(c->arena + L.off_aux + L.aux_bytes) : nullptr;
+  c->aux[0] = L.aux_bytes && c->arena_bytes >= L.total ? reinterpret_cast<float*>(c->arena + L.off_aux) : nullptr;
+  c->aux[1] = c->aa ? reinterpret_cast<float*>(c->arena + L.off_aux + L.aux_bytes) : nullptr;
   c->comp = L.comp_bytes ? reinterpret_cast<float*>(c->arena + L.off_comp) : nullptr;
 }
 
@@ -442,7 +445,7 @@ cudaError_t launch_step(hlbm_ctx* c, StepArgs a, bool moments) {
     }
     return launch_step_d3q39(a, c->kind, c->storage, moments, c->rows, c->npt, tm, c->stream);
   }
-  if (!moments && c->kind == KIND_SC && c->auto_schedule && !c->debug_skip_tma &&
+  if (!moments && c->kind == KIND_SC && c->aux[0] && c->auto_schedule && !c->debug_skip_tma &&
       two_launch_d2q37(c->storage, c->nx, c->ny, c->tma_ok)) {
     a.aux_wr = c->aux[0];
     a.aux_rd = c->aux[0];
@@ -718,7 +721,7 @@ hlbm_status hlbm_bind_memory(hlbm_ctx* c, void* dev_ptr, size_t bytes) {
   if (c->arena) return fail(c, HLBM_ESTATE, "memory already allocated or bound");
   if ((reinterpret_cast<uintptr_t>(dev_ptr) & 255) != 0) return fail(c, HLBM_EINVAL, "memory must be 256-byte aligned");
   const Layout L = layout(c->lattice, c->nx, c->ny, c->nz, &c->p);
-  if (bytes < L.total) return fail(c, HLBM_ENOMEM, "bound memory smaller than hlbm_workspace_bytes()");
+  if (bytes < L.required) return fail(c, HLBM_ENOMEM, "bound memory smaller than hlbm_workspace_bytes()");
   c->arena = static_cast<char*>(dev_ptr);
   c->arena_bytes = bytes;
   c->own_arena = false;

@@ -749,7 +749,8 @@ def main():
                          "algorithmic_bytes_per_node": bytes_per_node,
                          "kernel": "wall_complete_kernel + wall_moments_kernel + wall_collide_kernel (three launches per step, the "
                                    "populations read in both)" if case.params.get("walls") else
-                                   "aa_step_kernel (in place, one launch per step)" if case.params.get("lag") else
+                                   "aa_persistent_kernel or aa_step_kernel, by size (in place, one launch per step)"
+                                   if case.params.get("lag") else
                                    "the library's choice by size, kind and alignment" if not any(sched) else
                                    (("step3d_rows_kernel" if sched[2] >= 2 and case.nx in (32, 64, 128, 256)
                                      else "step3d_kernel") if case.lattice == "D3Q39" else

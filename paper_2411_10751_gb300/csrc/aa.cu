@@ -47,12 +47,12 @@ constexpr int frame_of() {
 // lanes (float2), rounding exactly like the one-node form.
 // aux: the neighbour field on the tile and its frame (shared memory).  sp: null,
 // or the tile's populations staged by TMA as Cfg2<ST, KIND_LOCAL> lays them out
-// (population i of the tile shifted by -c_i on odd steps); ready() returns once
-// they have landed, and staged_done() is called after a barrier once they are
-// all in registers.
-template <int ST, int KIND, bool ODD, bool MOM, int NPT, class Ready, class Done>
+// (population i of the tile shifted by -c_i on odd steps) and landed;
+// staged_done() is called once they are all in registers (after a barrier where
+// they were staged).
+template <int ST, int KIND, bool ODD, bool MOM, int NPT, class Done>
 __device__ __forceinline__ void aa_tile(const StepArgs& a, float* aux, const typename Codec<ST>::T* sp, int x0, int y0,
-                                        Ready&& ready, Done&& staged_done) {
+                                        Done&& staged_done) {
   using T = typename Codec<ST>::T;
   using V = typename std::conditional<NPT == 2, float2, float>::type;
   using Cf = Cfg2<ST, KIND_LOCAL, false, kBY>;
@@ -82,7 +82,6 @@ __device__ __forceinline__ void aa_tile(const StepArgs& a, float* aux, const typ
       aux[k] = __ldg(a.aux_rd + HLBM_IDX((long long)Y * nx + X, a.N, DBG_AUX));
     }
   }
-  ready();
   if (H > 0 || sp) __syncthreads();
 
   // the nodes' populations at time t
@@ -98,26 +97,26 @@ __device__ __forceinline__ void aa_tile(const StepArgs& a, float* aux, const typ
     __syncthreads();
     staged_done();
   } else {
-  int xs[7], ys[NPT][7];
+    int xs[7], ys[NPT][7];
 #pragma unroll
-  for (int d = -3; d <= 3; ++d) {
-    xs[d + 3] = wrap1(xc - d, nx);
+    for (int d = -3; d <= 3; ++d) {
+      xs[d + 3] = wrap1(xc - d, nx);
 #pragma unroll
-    for (int k = 0; k < NPT; ++k) ys[k][d + 3] = wrap1(yck[k] - d, ny) * nx;
-  }
-  static_for<37>([&](auto I) {
-    constexpr int i = I;
-#pragma unroll
-    for (int k = 0; k < NPT; ++k) {
-      if constexpr (!ODD) {
-        set_lane(g[i], k, to_float((f + (size_t)i * N)[(unsigned)HLBM_IDX(nodek[k], a.N, DBG_GATHER)]));
-      } else {
-        constexpr int cx = L::c(i, 0), cy = L::c(i, 1), b = aa_opp(i);
-        set_lane(g[i], k, to_float((f + (size_t)b * N)[(unsigned)HLBM_IDX(ys[k][cy + 3] + xs[cx + 3], a.N, DBG_GATHER)]));
-      }
+      for (int k = 0; k < NPT; ++k) ys[k][d + 3] = wrap1(yck[k] - d, ny) * nx;
     }
-  });
-  staged_done();
+    static_for<37>([&](auto I) {
+      constexpr int i = I;
+#pragma unroll
+      for (int k = 0; k < NPT; ++k) {
+        if constexpr (!ODD) {
+          set_lane(g[i], k, to_float((f + (size_t)i * N)[(unsigned)HLBM_IDX(nodek[k], a.N, DBG_GATHER)]));
+        } else {
+          constexpr int cx = L::c(i, 0), cy = L::c(i, 1), b = aa_opp(i);
+          set_lane(g[i], k, to_float((f + (size_t)b * N)[(unsigned)HLBM_IDX(ys[k][cy + 3] + xs[cx + 3], a.N, DBG_GATHER)]));
+        }
+      }
+    });
+    staged_done();
   }
 
   V dr, dr_l, acc, J[3], Pih;
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(kBX * kBY / NPT, 2 * NPT) aa_step_kernel(const
   constexpr int H = frame_of<KIND>();
   __shared__ float aux[(H > 0) ? (kBX + 2 * H) * (kBY + 2 * H) : 1];
   grid_dependency_wait();
-  aa_tile<ST, KIND, ODD, MOM, NPT>(a, aux, nullptr, blockIdx.x * kBX, blockIdx.y * kBY, [] {}, [] {});
+  aa_tile<ST, KIND, ODD, MOM, NPT>(a, aux, nullptr, blockIdx.x * kBX, blockIdx.y * kBY, [] {});
 }
 
 // Persistent CTAs, two nodes per thread, that stage the next tile's populations
@@ -370,7 +369,7 @@ __global__ void __launch_bounds__(kBX * kBY / 2, 4)
       }
       phase ^= 1u;
     }
-    aa_tile<ST, KIND, ODD, false, 2>(a, aux, boxed ? sp : nullptr, x0, y0, [] {}, [&] {
+    aa_tile<ST, KIND, ODD, false, 2>(a, aux, boxed ? sp : nullptr, x0, y0, [&] {
       if ((tid & 31) == 0) stage(tn);
       if (tid == 0 && tn < ntiles) raw = atomicAdd(a.tile_ctr, 1ull);
     });

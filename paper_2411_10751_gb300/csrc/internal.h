@@ -39,11 +39,13 @@ int per_device_cached(std::atomic<int> (&cache)[kMaxDevicesCached], F&& compute)
   return n;
 }
 
-// Launches a kernel that may start while the launch before it on the stream
-// still runs (programmatic dependent launch, also inside a captured graph):
-// its blocks take free slots and run up to grid_dependency_wait()
-// (step_common.cuh) meanwhile.  The kernel must execute that wait before its
-// first access to memory that an earlier launch reads or writes.  A refused
+// Launches a kernel dependently on the launch before it on the stream
+// (programmatic dependent launch, also inside a captured graph).  No kernel here
+// lets its dependents in early, so its blocks start once every block of the launch
+// before has ended, and what overlaps is the launch's latency and the flush of that
+// launch's writes, which grid_dependency_wait() (step_common.cuh) waits for.  The
+// kernel must execute that wait before its first access to memory that an earlier
+// launch reads or writes.  A refused
 // launch is this call's result only: the thread's last error is taken back, or the
 // next launch of another context would report it.
 template <class... P>

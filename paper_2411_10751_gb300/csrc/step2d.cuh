@@ -99,24 +99,20 @@ __device__ __forceinline__ void load_region(const typename Cf::T* sp, int rx, in
   });
 }
 
-// theta - 1 of a node from its moments (Eq. 4.5), local force only
-template <class L>
-__device__ __forceinline__ float theta_bar_of(const StepArgs& a, float dr, float J0, float J1, float Pih, int node, int y) {
-  const float rho = a.rho0 + dr;
-  float gacc[3];
-  accel<2>(a, node, y, gacc);
-  const float inv = rcp_nr(rho);
-  const float ux = fmaf(0.5f * rho, gacc[0], J0) * inv;
-  const float uy = fmaf(0.5f * rho, gacc[1], J1) * inv;
-  const float G2 = 2.f * rho * (ux * gacc[0] + uy * gacc[1]);
-  constexpr float Dc = (float)(2.0 * L::cs2);
-  return (Pih - rho * (ux * ux + uy * uy) + 0.5f * G2) * inv * (1.f / Dc);
-}
+// theta - 1 of a node from its pulled populations (Eq. 4.5), local force only
 template <class L>
 __device__ __forceinline__ float theta_bar_local(const StepArgs& a, float (&g)[L::Q], int node, int y) {
   float dr, acc, J[3], Pih;
   moments_h<L>(g, dr, acc, J, Pih);
-  return theta_bar_of<L>(a, dr, J[0], J[1], Pih, node, y);
+  const float rho = a.rho0 + dr;
+  float gacc[3];
+  accel<2>(a, node, y, gacc);
+  const float inv = rcp_nr(rho);
+  const float ux = fmaf(0.5f * rho, gacc[0], J[0]) * inv;
+  const float uy = fmaf(0.5f * rho, gacc[1], J[1]) * inv;
+  const float G2 = 2.f * rho * (ux * gacc[0] + uy * gacc[1]);
+  constexpr float Dc = (float)(2.0 * L::cs2);
+  return (Pih - rho * (ux * ux + uy * uy) + 0.5f * G2) * inv * (1.f / Dc);
 }
 
 // CTAs per SM the register budget is sized for: as many as the staged tile's

@@ -155,9 +155,7 @@ struct CompShared {
   double v[24][32];              // values that the four warps exchange, per lane
 };
 
-__device__ __forceinline__ void comp_barrier() { asm volatile("barrier.sync 2, 128;" ::: "memory"); }
-
-// Called by four whole warps (wq = 0 .. 3).  x0: first column of the block.
+// Called by the block's four warps (wq = 0 .. 3).  x0: first column of the block.
 __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, int x0, int wq, int lane, const CompIn& in,
                                                  CompShared& sh) {
   const int lc = lane / 6, t = lane - 6 * lc;
@@ -204,7 +202,7 @@ __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, in
       sh.v[o + 3][lane] = fma(hb4, m[4], T);
     }
   }
-  comp_barrier();
+  __syncthreads();
   // phase 2: R_a of each state, and the sums over the row's velocities of w (P - 1)
   if (!(wq & 1)) {
     const int o = wq == 0 ? TT : TP, d = wq == 0 ? RT : RP;
@@ -215,7 +213,7 @@ __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, in
     sh.v[d + 3][lane] = m[4];
     sh.v[d + 4][lane] = fma(w4, m[4], fma(w2, r2, __dmul_rn(w0, sh.v[o + 3][lane])));
   }
-  comp_barrier();
+  __syncthreads();
   // phase 3: s - 1 = sum_rows (B - A) / sum_rows (W + A), and beside it the differences
   double x1 = 0.0, d1 = 0.0, x2 = 0.0, d2 = 0.0;
   if (wq == 3) {
@@ -240,7 +238,7 @@ __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, in
     x2 = sh.v[RT + i + 2][lane];
     d2 = __dsub_rn(x2, sh.v[RP + i + 2][lane]);
   }
-  comp_barrier();
+  __syncthreads();
   // phase 4: T' and R'_a
   if (wq != 3) {
     const double sm1 = sh.v[SM1][lane];
@@ -251,7 +249,7 @@ __device__ __forceinline__ void complete_columns(const WallArgs& a, int side, in
       sh.v[RPR + wq + 1][lane] = fma(sm1, x2, d2);
     }
   }
-  comp_barrier();
+  __syncthreads();
   const double rp = p[0];
   // phase 5: the velocities (+-cx, k), cx = wq: g_i = g*_ibar + rho_p (s P_i - P_ibar)
   const int x = x0 + col;

@@ -316,13 +316,14 @@ bool auto_rows3(const hlbm_ctx* c, double bytes) {
 // staged tiles, D3Q39 whole rows).  Their CTAs take ordered tiles and hold the
 // next one in flight, which pays once a step streams from HBM, i.e. when the two
 // buffers outgrow what L2 (129 MB) keeps of them; inside it the hardware's own
-// block scheduling is faster.  us per step, one CTA per tile against
-// persistent, FP32 unless stated: thermal 512 x 512 (78 MB) 16.7 / 18.0, 576 x 576
-// (98 MB) 21.4 / 19.6, 1024 x 1024 60.9 / 54.9; pseudopotential 576 x 576 35.9 /
-// 34.8, 1024 x 1024 95.5 / 89.4 (D3Q39 above).  Not for D2Q37 in 16 bits, whose persistent form has 3
-// CTAs per SM instead of 4 (thermal 1024 x 1024 45.4 / 48.8), nor for the body
-// force alone, which gains at some sizes (1024 x 1024 54.1 / 53.1) and loses at
-// others (1536 x 1536 109.1 / 112.4).
+// block scheduling is faster.  us per step, one CTA per tile against persistent,
+// FP32 unless stated: thermal 512 x 512 (78 MB) 16.6 / 18.4, 576 x 576 (98 MB) 21.1 /
+// 19.3, 1024 x 1024 61.1 / 55.3; pseudopotential 576 x 576 35.2 / 34.2, 1024 x 1024
+// 94.7 / 89.4 (D3Q39 above).  Not for D2Q37 in 16 bits, whose persistent form has 3
+// CTAs per SM instead of 4 (1024 x 1024 thermal 45.1 / 48.6, pseudopotential 64.9 /
+// 71.5), nor for the body force alone, which gains at some sizes (1024 x 1024 54.7 /
+// 53.4, FP16 40.6 / 38.6) and loses at others (608 x 608 18.5 / 20.3, 1536 x 1536 111.2 /
+// 113.2).
 int auto_persistent(const hlbm_ctx* c) {
   const double bytes = 2.0 * c->Q * (double)c->N * (double)c->elem;
   if (bytes < 96e6) return 0;

@@ -13,8 +13,11 @@
 // are read from device memory one item ahead, by the last warps while the
 // others collide.  It is bound by instruction issue (half of the slots) and the
 // loads' latency at 22 warps per SM: 256 domains, 6.4 M nodes, FP32, 770 us a step
-// staged, 564 us pulled, 515 us with 32-bit offsets in the pulls.  Three CTAs per
-// SM at 56 registers took 643 us.
+// staged, 564 us pulled, 522 us with 32-bit offsets in the pulls (FP16 484; three
+// CTAs per SM at 56 registers 559 and 509).  Batches of large aligned domains gain
+// less, since their tiles could be staged (us per step, staged / pulled, four
+// domains of 1024 x 1024: thermal 325 / 273, body force 304 / 243, pseudopotential
+// 379 / 383; of 512 x 512 90.6 / 72.6 thermal, 106 / 99.9 pseudopotential).
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -199,7 +202,7 @@ hlbm_status hlbm_batch_create(int n, hlbm_ctx* const* ctxs, hlbm_batch** out) {
 static hlbm_status batch_refresh(hlbm_batch* b) {
   b->host.assign(b->ctxs.size(), BatchDomain{});
   b->items.clear();
-  std::vector<BatchItem> heavy, light;   // pseudopotential tiles (compute-bound) and the others (HBM-bound)
+  std::vector<BatchItem> heavy, light;   // pseudopotential tiles (the longest) and the others
   for (int kind : {(int)KIND_SC, (int)KIND_THERMAL, (int)KIND_LOCAL}) {
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
       hlbm_ctx* c = b->ctxs[k];
@@ -215,8 +218,8 @@ static hlbm_status batch_refresh(hlbm_batch* b) {
         for (int x0 = 0; x0 < nx; x0 += 32) (dkind == KIND_SC ? heavy : light).push_back(BatchItem{(int)k, dkind, x0, y0});
     }
   }
-  // the slow tiles first, so the launch ends on short ones (measured against
-  // spreading them evenly among the others: 8.30k vs 8.22k MLUPS)
+  // the slow tiles first, so the launch ends on short ones (against spreading them
+  // evenly among the others, 256 domains, us per step: FP16 484 / 493, FP32 522 / 509)
   b->items = heavy;
   b->items.insert(b->items.end(), light.begin(), light.end());
   if (b->grid == 0)

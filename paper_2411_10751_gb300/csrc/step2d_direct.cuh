@@ -179,12 +179,15 @@ __global__ void __launch_bounds__(Direct2<KIND>::NT, PER) step2d_direct_kernel(c
   direct_tile<ST, KIND, D::NT>(a, aux, blockIdx.x * D::BX, blockIdx.y * D::BY);
 }
 
-// Blocks per SM of the throughput form: 80 registers leave 2 thermal and 3
-// body-force blocks (3 and 4, with 56 and 64 registers, spill and gain nothing:
-// 901 x 899 58.2 against 58.5 us, 47.3 against 48.3 us); the pseudopotential
-// block of 17 warps at 56 registers with 100 B of spills pays off as soon as
-// the tiles outnumber the SMs (641 x 639 FP32 52.0 -> 45.9 us; on fewer tiles
-// one block per SM without spills: 64 x 64 5.0 -> 4.4 us).
+// Blocks per SM that the registers are sized for (us per step): 80 registers
+// leave 2 thermal and 3 body-force blocks; one more of each, with 56 and 64
+// registers, spills and is slower on small domains and in 16 bits (thermal 64 x 64
+// 3.20 / 3.34, 256 x 256 FP16 5.0 / 5.5, 901 x 899 FP16 46.4 / 46.9) but faster on large
+// FP32 ones (901 x 899 thermal 55.9 / 51.9, body force 48.9 / 47.9).  The
+// pseudopotential block of 17 warps takes 56 registers and 100 B of spills for two
+// blocks as soon as the tiles outnumber the SMs (one / two per SM: 256 x 256 7.7 /
+// 7.1, 64 x 64 4.0 / 4.3).  Reading psi from its field, three against two: 901 x 899
+// 78.0 / 88.4.
 template <int KIND>
 constexpr int direct2_per_sm() {
   return KIND == KIND_LOCAL || KIND == KIND_SCF ? 3 : 2;

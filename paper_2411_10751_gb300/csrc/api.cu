@@ -294,22 +294,23 @@ constexpr double kMinBoxed = 0.62;
 
 // Whether a D3Q39 context without a schedule runs the whole-row kernel.  Planes
 // whose rows cross the y-edge are copied row by row, which costs most where a tile
-// has many rows (8 at nx = 32, 4 at nx = 64) of a small ny; what it saves most on is
-// a force field, which it stages beside them.  us per step, gather kernel / whole
-// rows.  nx = 32, FP32, field: 32 x 7 x 1600 21.8 / 43.0, 32 x 24 x 900 41.9 / 39.3,
-// 32 x 101 x 99 (100 MB) 17.0 / 21.7, 32 x 64 x 180 (115 MB) 20.9 / 20.3, 32 x 160 x
-// 160 49.1 / 40.7; no field: 32 x 300 x 60 31.2 / 31.9, 32 x 160 x 160 41.5 / 40.0.
-// nx = 64, FP32, field: 64^3 (82 MB) 12.4 / 14.1, 64 x 64 x 80 (102 MB) 17.8 / 16.7; no
-// field: 64 x 64 x 80 14.9 / 16.6, 64 x 64 x 100 (128 MB) 21.4 / 19.7, 64 x 9 x 1200
-// 46.1 / 47.7, 64 x 16 x 700 37.1 / 35.5.  nx >= 128, FP32, no field: 128 x 50 x 50 (100
-// MB) 15.8 / 15.3, 128 x 7 x 600 30.4 / 28.1, 128^3 100.6 / 94.7 (field 120.0 / 98.8).  FP16, field:
-// 64 x 64 x 160 (102 MB) 31.0 / 29.2; no field: 28.5 / 29.4, 64 x 128 x 128 (164 MB) 44.4 /
-// 43.1.
+// has many rows (8 at nx = 32, 4 at nx = 64) of a small ny, and tiles that end past
+// ny work for nothing; what it saves most on is a force field, which it stages
+// beside them.  us per step, gather kernel / whole rows.  nx = 32, FP32, field: 32 x
+// 7 x 1600 21.8 / 43.0, 32 x 24 x 900 41.9 / 39.3, 32 x 101 x 99 (100 MB) 17.0 / 21.7,
+// 32 x 64 x 180 (115 MB) 20.9 / 20.3, 32 x 160 x 160 49.1 / 40.7; no field: 32 x 128 x
+// 90 (115 MB) 17.4 / 19.1, 32 x 40 x 560 37.0 / 37.6, 32 x 56 x 400 (224 MB) 37.0 /
+// 36.6, 32 x 160 x 160 41.7 / 39.7, 32 x 164 x 160 43.3 / 45.2.  nx = 64, FP32, field:
+// 64^3 (82 MB) 12.4 / 14.1, 64 x 64 x 80 (102 MB) 17.8 / 16.7; no field: 64 x 64 x 80
+// 14.9 / 16.6, 64 x 64 x 100 (128 MB) 21.4 / 19.7, 64 x 9 x 1200 46.1 / 47.7, 64 x 16 x
+// 700 37.1 / 35.5; FP16, field: 64 x 64 x 160 (102 MB) 31.0 / 29.2; no field: 28.5 /
+// 29.4, 64 x 128 x 128 (164 MB) 44.4 / 43.1.  nx >= 128, no field: 128 x 50 x 50 (100 MB)
+// 15.8 / 15.3, 128 x 7 x 600 30.4 / 28.1, 128^3 100.6 / 94.7 (field 120.0 / 98.8), FP16
+// 128 x 75 x 64 (96 MB) 27.9 / 26.9, 256 x 40 x 64 (102 MB) 28.5 / 27.7.
 bool auto_rows3(const hlbm_ctx* c, double bytes) {
   const bool field = c->force_mode == FORCE_FIELD, tall = c->ny >= 3 * (256 / c->nx);
-  if (c->nx == 32) return field && tall && bytes >= 112e6;
-  if (field || (c->storage == ST_F32 && c->nx >= 128)) return bytes >= 96e6;
-  return tall && bytes >= 120e6;
+  if (c->nx == 32) return field ? tall && bytes >= 112e6 : c->ny % 8 == 0 && c->ny >= 56 && bytes >= 200e6;
+  return field || c->nx >= 128 ? bytes >= 96e6 : tall && bytes >= 120e6;
 }
 
 // Whether a context without a schedule runs the persistent kernels (D2Q37
